@@ -416,7 +416,8 @@ cudaError_t launch_opacity_p(const FwdParams& p, const CUtensorMap& sig, const C
 // per CTA (item-major, so consecutive units of a CTA mostly share the item and its path
 // lengths).  A producer warp loads each unit's K tile [N][kTW] by 2-D TMA boxes of kCB rows
 // into one of up to three tile slots, plus the item's packed path lengths and annulus weights by
-// bulk copy when the item changes (after every earlier unit is done with them).  The W
+// bulk copy when the item changes (after every earlier unit is done with them), on a barrier of
+// their own: a K tile of the item's second unit can land before them.  The W
 // contraction warps take work items (unit, 16-ray tile) from a shared counter, a unit's longest
 // tile first: tau = DL K for the tile's rays and its partial depth sum_j a_j (1 - e^-tau_j),
 // stored per tile.  The warp that completes a unit's last tile adds the tiles' partials in
@@ -455,7 +456,7 @@ __global__ void __launch_bounds__(32 * (W + 1), 1)
 k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, long long kcols, int Bc,
                 int n_tiles, int n_slots) {
   extern __shared__ unsigned char csm_raw[];
-  __shared__ __align__(8) uint64_t kfull[kMaxSlots], kempty[kMaxSlots];
+  __shared__ __align__(8) uint64_t kfull[kMaxSlots], kempty[kMaxSlots], dlfull;
   __shared__ int abort_flag, next_item, done[kMaxSlots], slot_unit[kMaxSlots];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const ContractLayout lay(p.max_layers, n_slots);
@@ -469,6 +470,7 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, long long
       done[i] = 0;
       slot_unit[i] = i;                                 // units 0 .. S-1 go to slots 0 .. S-1
     }
+    mbar_init(&dlfull, 1);
     abort_flag = 0;
     next_item = 0;
     mbar_fence_init();
@@ -487,7 +489,7 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, long long
   if (warp == W) {
     // ---------------- producer
     if (lane != 0) return;
-    int dl_item = -1;
+    int dl_item = -1, dl_phases = 0;                    // dlfull: one phase per item
     int k = 0;
     for (; k < n_units; ++k) {
       const int u = u_begin + k;
@@ -496,30 +498,35 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, long long
       const int N = p.buf.items[b].n_layers;
       const int sl = k % S, q = k / S;
       bool ok = q == 0 || mbar_wait_bounded(&kempty[sl], (q - 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
-      const bool new_item = N > 0 && b != dl_item;
+      const bool new_item = b != dl_item;
       // the units in the other slots must be done with the path lengths too
       for (int d = 1; ok && new_item && d < S && d <= k; ++d) {
         const int kp = k - d;
         ok = mbar_wait_bounded(&kempty[kp % S], (kp / S) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
       }
       if (!ok || *(volatile int*)&abort_flag) { atomicExch(&abort_flag, 1); break; }
+      if (new_item) {
+        dl_item = b;
+        ++dl_phases;
+        if (N == 0) {
+          mbar_arrive(&dlfull);
+        } else {
+          mbar_arrive_expect_tx(&dlfull, (uint32_t)(dlp_offset(N) * 4 + p.buf.npad * 4));
+          bulk_g2s(DLP, p.buf.dlp + (size_t)b * dlp_offset(p.max_layers),
+                   (uint32_t)(dlp_offset(N) * 4), &dlfull);
+          bulk_g2s(a_s, p.buf.aj + (size_t)b * p.buf.npad, (uint32_t)(p.buf.npad * 4), &dlfull);
+        }
+      }
       if (N == 0) { mbar_arrive(&kfull[sl]); continue; }   // nothing to load
       const int nbox = (N + kCB - 1) / kCB;
-      uint32_t bytes = (uint32_t)nbox * kCB * kTW * 4;
-      if (new_item) bytes += (uint32_t)(dlp_offset(N) * 4 + p.buf.npad * 4);
-      mbar_arrive_expect_tx(&kfull[sl], bytes);
+      mbar_arrive_expect_tx(&kfull[sl], (uint32_t)nbox * kCB * kTW * 4);
       float* Kt = reinterpret_cast<float*>(base + sl * lay.slot);
       for (int i = 0; i < nbox; ++i)
         tma_load_2d(Kt + (size_t)i * kCB * kTW, &tm_k, tile * kTW, bc * p.max_layers + i * kCB,
                     &kfull[sl]);
-      if (new_item) {
-        bulk_g2s(DLP, p.buf.dlp + (size_t)b * dlp_offset(p.max_layers),
-                 (uint32_t)(dlp_offset(N) * 4), &kfull[sl]);
-        bulk_g2s(a_s, p.buf.aj + (size_t)b * p.buf.npad, (uint32_t)(p.buf.npad * 4), &kfull[sl]);
-        dl_item = b;
-      }
     }
     // every copy issued has landed before the CTA may exit
+    if (dl_phases > 0) mbar_wait_bounded(&dlfull, (dl_phases - 1) & 1, nullptr, 0);
     for (int i = 0; i < S && i < k; ++i) {
       const int kl = k - 1 - i;
       mbar_wait_bounded(&kfull[kl % S], (kl / S) & 1, nullptr, 0);
@@ -546,9 +553,13 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, long long
     const int sl = k % S, q = k / S;
     // the slot holds unit k - S until that unit's last tile hands it over; only then is
     // phase q the one kfull[sl] is in (a warp may take work of later units early)
+    // then the item's path lengths: dlfull's phase is the item's ordinal in this CTA, and the
+    // next item's starts only when every unit of this one is done
     const bool ok = __all_sync(0xffffffffu, wait_slot(&slot_unit[sl], k, &abort_flag, p.dev_err) &&
                                                 mbar_wait_bounded(&kfull[sl], q & 1, p.dev_err,
                                                                   TR_DEVERR_TIMEOUT) &&
+                                                mbar_wait_bounded(&dlfull, (bc - u_begin / n_tiles) & 1,
+                                                                  p.dev_err, TR_DEVERR_TIMEOUT) &&
                                                 !*(volatile int*)&abort_flag);
     if (!ok) { if (lane == 0) atomicExch(&abort_flag, 1); return; }
     float* part = reinterpret_cast<float*>(base + sl * lay.slot + lay.ktb);
