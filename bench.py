@@ -671,8 +671,8 @@ def algorithmic_bytes(tb, atm, kernel: str = "method") -> int:
 
 CSRC = os.path.join(ROOT, "paper_1912_07759_gb300", "csrc")
 KERNEL_SOURCES = {  # the files each kernel is built from (its ncu summary records their hash)
-    "k_opacity_fp32": ["forward_fp32.cu", "opacity.h", "tma.h", "tr_internal.h"],
-    "k_opacity_fp16": ["forward_fp32.cu", "opacity.h", "tma.h", "tr_internal.h"],
+    "k_opacity_fp32": ["opacity_rows.cu", "opacity.h", "tma.h", "tr_internal.h"],
+    "k_opacity_fp16": ["opacity_rows.cu", "opacity.h", "tma.h", "tr_internal.h"],
     "k_contract_fp32": ["forward_fp32.cu", "tma.h", "tr_internal.h"],
     "k_contract_tc": ["tc_fp32.cu", "umma.h", "tma.h", "tr_internal.h"],
     "k_contract_umma": ["mixed.cu", "umma.h", "tma.h", "tr_internal.h"],

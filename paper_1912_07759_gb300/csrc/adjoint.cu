@@ -236,10 +236,10 @@ k_adjoint_tile(AdjParams a) {
   const bool in_row = w2 < p.wn_pad;
   const LayerDesc* LD = p.buf.layers + (size_t)b * p.max_layers;
   if constexpr (!RECOMP) {
-    const float* ks = a.kstore + (size_t)b * p.max_layers * a.kcols + (size_t)(a.tile0 + tile) * kAT + 2 * lane;
+    const float* ks = a.kstore + k_index(b, (long long)(a.tile0 + tile) * kAT + 2 * lane, 0, a.kcols, p.max_layers);
     for (int l = warp; l < N; l += kAWarps)
       *reinterpret_cast<float2*>(Kt + tix(l, 2 * lane)) =
-          __ldg(reinterpret_cast<const float2*>(ks + (size_t)l * a.kcols));
+          __ldg(reinterpret_cast<const float2*>(ks + (size_t)l * kKTile));
   } else {
     // K recomputed with the opacity kernel's arithmetic, so that it equals the stored K bit
     // for bit: per (P, T) cell the molecule sums us_c = sum_m (x_m / x_max) sigma_m,c and per

@@ -461,6 +461,15 @@ static bool encode_table_map(CUtensorMap* m, const void* base, bool fp16, int wn
 static bool encode_tables(tr_tables* t) {
   if (t->n_mol > 0) {
     const int dims[3] = {t->n_t, t->n_p, t->n_mol}, box[3] = {2, 2, t->n_mol};
+    const int box_t[3] = {2, 1, t->n_mol}, box_p[3] = {1, 2, t->n_mol};
+    if (t->d_sigma &&
+        (!encode_table_map(&t->tm_row_t32, t->d_sigma, false, t->wn_pad, 4, dims, box_t, kRowTile) ||
+         !encode_table_map(&t->tm_row_p32, t->d_sigma, false, t->wn_pad, 4, dims, box_p, kRowTile)))
+      return false;
+    if (t->d_logsig16 &&
+        (!encode_table_map(&t->tm_row_t16, t->d_logsig16, true, t->wn_pad, 4, dims, box_t, kRowTile) ||
+         !encode_table_map(&t->tm_row_p16, t->d_logsig16, true, t->wn_pad, 4, dims, box_p, kRowTile)))
+      return false;
     if (t->d_sigma &&
         (!encode_table_map(&t->tm_sig32, t->d_sigma, false, t->wn_pad, 4, dims, box, kOpacityTile) ||
          !encode_table_map(&t->tm_sig32_f, t->d_sigma, false, t->wn_pad, 4, dims, box, kFusedTile)))
@@ -470,8 +479,9 @@ static bool encode_tables(tr_tables* t) {
       return false;
   }
   if (t->n_cia > 0) {
-    const int dims[2] = {t->n_t_cia, t->n_cia}, box[2] = {2, t->n_cia};
-    if (!encode_table_map(&t->tm_cia, t->d_cia, false, t->wn_pad, 3, dims, box, kOpacityTile) ||
+    const int dims[2] = {t->n_t_cia, t->n_cia}, box[2] = {2, t->n_cia}, box_r[2] = {1, t->n_cia};
+    if (!encode_table_map(&t->tm_row_cia, t->d_cia, false, t->wn_pad, 3, dims, box_r, kRowTile) ||
+        !encode_table_map(&t->tm_cia, t->d_cia, false, t->wn_pad, 3, dims, box, kOpacityTile) ||
         !encode_table_map(&t->tm_cia_f, t->d_cia, false, t->wn_pad, 3, dims, box, kFusedTile))
       return false;
   }
@@ -948,29 +958,37 @@ int tr::run_forward(tr_ctx* ctx, const tr_tables* t, int max_layers, const ItemB
     if (e == cudaSuccess) e = tiles_kernel(s);
     if (e != cudaSuccess) return cuda_fail(ctx, e, "path-length kernels");
   }
-  // two stages per chunk of items: opacity -> K in kbuf -> contraction + depth
-  const int chunk = forward_chunk_items(B, max_layers, wn_begin, wn_count);
-  for (int b0 = 0; b0 < B && e == cudaSuccess; b0 += chunk) {
-    const int bc = std::min(chunk, B - b0);
-    p.b_off = b0;
-    {
-      KernelTimer kt(ctx, mixed ? "k_opacity_fp16" : "k_opacity_fp32", s);
-      e = launch_opacity(p, mixed ? &t->tm_sig16 : &t->tm_sig32, &t->tm_cia, bc, kbuf,
-                         choice ? choice->per_sm : 0, s);
+  // two stages per part of the work that fits the K buffer: opacity -> K in kbuf -> contraction
+  // + depth
+  const KSplit ks = opacity_only ? KSplit{B, (int)forward_kcols(wn_begin, wn_count)}
+                                 : forward_split(B, max_layers, wn_begin, wn_count);
+  const int w_end = wn_begin + wn_count;
+  bool first = true;
+  for (int b0 = 0; b0 < B && e == cudaSuccess; b0 += ks.items)
+    for (int w0 = wn_first(wn_begin); w0 < w_end && e == cudaSuccess; w0 += ks.cols) {
+      const int bc = std::min(ks.items, B - b0);
+      p.b_off = b0;
+      p.wn_begin = std::max(w0, wn_begin);
+      p.wn_count = std::min(w0 + ks.cols, w_end) - p.wn_begin;
+      p.out = out ? out + (p.wn_begin - wn_begin) : nullptr;
+      {
+        KernelTimer kt(ctx, mixed ? "k_opacity_fp16" : "k_opacity_fp32", s);
+        e = launch_opacity(p, t, bc, kbuf, choice ? choice->per_sm : 0, s);
+      }
+      if (e != cudaSuccess || opacity_only) break;
+      if (branch && first) {
+        // the path lengths and their tiles beside the opacity kernel, then the join
+        e = fork_start(ctx, fork, s, true);
+        if (e == cudaSuccess) e = tiles_kernel(fork->aux);
+        join_fork(ctx, fork, s);
+        if (e != cudaSuccess) break;
+      }
+      first = false;
+      KernelTimer kt(ctx, mixed ? "k_contract_umma" : kind == kContractTC ? "k_contract_tc"
+                                                                          : "k_contract_fp32", s);
+      e = mixed ? launch_contract_umma(p, bc, kbuf, dl16, s)
+                : launch_contract_fp32(p, bc, kbuf, kind, dl16, s);
     }
-    if (e != cudaSuccess || opacity_only) break;
-    if (branch && b0 == 0) {
-      // the path lengths and their tiles beside the opacity kernel, then the join
-      e = fork_start(ctx, fork, s, true);
-      if (e == cudaSuccess) e = tiles_kernel(fork->aux);
-      join_fork(ctx, fork, s);
-      if (e != cudaSuccess) break;
-    }
-    KernelTimer kt(ctx, mixed ? "k_contract_umma" : kind == kContractTC ? "k_contract_tc"
-                                                                        : "k_contract_fp32", s);
-    e = mixed ? launch_contract_umma(p, bc, kbuf, dl16, s)
-              : launch_contract_fp32(p, bc, kbuf, kind, dl16, s);
-  }
   return e == cudaSuccess ? TR_OK : cuda_fail(ctx, e, "forward kernels");
 }
 

@@ -33,7 +33,7 @@ constexpr double kC2cmK = 6.62607015e-34 * 299792458.0 / 1.380649e-23 * 100.0;
 struct EmParams {
   ItemBuffers buf;
   int max_layers;
-  const float* kbuf;            // K of the chunk: kbuf[(c * max_layers + l) * kcols + x]
+  const float* kbuf;            // K of the chunk (k_index)
   long long kcols;
   const double* wn;             // [n_wn] native wavenumbers (1/cm)
   int wn_begin, wn_count, b_off;
@@ -86,7 +86,7 @@ __global__ void __launch_bounds__(kEmThreads) k_emission(EmParams p) {
   if (N == 0) { *o = 0.0; return; }
   const int w = p.wn_begin + i;
   const float nu = (float)__ldg(p.wn + w);
-  const float* kr = p.kbuf + (size_t)c * p.max_layers * p.kcols + (w - wn_first(p.wn_begin));
+  const float* kr = p.kbuf + k_index(c, w - wn_first(p.wn_begin), 0, p.kcols, p.max_layers);
   float I[MU];
   const float bs = planck_shape(nu * (float)(kC2cmK / ig.t_surf));   // surface, E3
 #pragma unroll
@@ -102,7 +102,7 @@ __global__ void __launch_bounds__(kEmThreads) k_emission(EmParams p) {
     for (int k = 0; k < MU; ++k)
       if (k < p.n_mu) I[k] = fmaf(I[k] - bl, ex2f(dtau * p.mu_coef[k]), bl);
   };
-  const long long kc = p.kcols;
+  constexpr int kc = kKTile;                            // the next layer of the tile
   int l0 = 0;
   for (; l0 + kU <= N; l0 += kU, kr += kU * kc) {      // whole blocks, no per-layer guard
     float kv[kU];
@@ -212,7 +212,7 @@ int run_emission(tr_ctx* ctx, const tr_tables* t, int max_layers, const ItemBuff
     fp.b_off = b0;
     {
       KernelTimer kt(ctx, mixed ? "k_opacity_fp16" : "k_opacity_fp32", s);
-      e = launch_opacity(fp, mixed ? &t->tm_sig16 : &t->tm_sig32, &t->tm_cia, bc, kbuf, 0, s);
+      e = launch_opacity(fp, t, bc, kbuf, 0, s);
     }
     if (e != cudaSuccess) break;
     ep.b_off = b0;

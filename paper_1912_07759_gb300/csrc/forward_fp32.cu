@@ -1,12 +1,13 @@
 // forward_fp32.cu -- the two-stage forward form: opacity K[layer, wn] (Sec. 5 linear P/T
 // interpolation, weighted by rho X and fused with Rayleigh, CIA and the grey cloud as in
-// Sec. 8.1) streamed to HBM by k_opacity, then the slant optical depth
+// Sec. 8.1) streamed to HBM by k_opacity_rows (opacity_rows.cu; k_opacity_exp here for the
+// exponential temperature scheme), then the slant optical depth
 // tau[ray, wn] = sum_{l >= j} DL[j][l] K[l][wn] (Sec. 4, eqs. tot_opt_dpth, opt_dpth,
 // cia_opt_dpth) and transit depth D = (R_p/R_s)^2 + sum_j a_j (1 - exp(-tau_j)) (Sec. 4, eqs.
 // Delta_lambda, a_lambda) by k_contract_fp32 (FP32) or k_contract_umma (mixed.cu, tensor
-// cores).  Items are processed in chunks whose K fits a 2 GiB budget.  k_opacity stages the
-// bracketing table rows in shared memory by TMA tensor-map loads (opacity.h); with FP16 log
-// tables it decodes them on the fly.  This is the default form of both precisions when a K
+// cores).  The work is cut into parts whose K fits a 2 GiB budget.  Both opacity kernels stage
+// the bracketing table rows in shared memory by TMA tensor-map loads and decode FP16 log tables
+// on the fly.  This is the default form of both precisions when a K
 // buffer is available; the fused kernel (fused.cu) serves callers without one.
 //
 // The FP32 contraction: a warp takes one 16-ray register tile (j0..j0+15) of a unit at a time, a
@@ -95,17 +96,17 @@ __device__ __forceinline__ void contract_tile(int N, int j0, const float* Kt, co
   }
 }
 
-// ---- TMA-staged opacity (first stage of the two-stage form, both table precisions)
+// ---- TMA-staged opacity with the exponential temperature scheme (first stage of the two-stage
+// form, both table precisions; the linear scheme's kernel is k_opacity_rows)
 //
 // Work unit = one item x kOT consecutive wavenumbers; a persistent grid of CTAs walks the units
 // (items vary fastest, so CTAs running together share a wavenumber tile's table rows in L2).
 // A producer warp streams each unit's segments through the ring of table-row stages
-// (opacity.h); kOCW consumer warps (two wavenumbers per lane) sum each segment's rows over
-// molecules and CIA pairs and form K of every layer of the segment from those sums:
-//   K = kappa_cloud + rho sigma_R + sum_c (rho x_max w_c) sum_m x_m sigma_m,c
+// (opacity.h); kOCW consumer warps (two wavenumbers per lane) take the logarithms of each
+// segment's rows and form K of every layer of the segment:
+//   K = kappa_cloud + rho sigma_R + sum_P (rho x_max w_P) sum_m x_m sigma_m,P(T)
 //         + sum_T (rho^2 y_max w_T) sum_q y_q sigma_q,T
-// with bilinear corner weights w_c and CIA temperature weights w_T (Sec. 5, Sec. 8.1).  K is
-// streamed to HBM once.  Both roles read the layers' brackets and coefficients 32 layers per
+// with the P weights w_P and CIA temperature weights w_T (Sec. 5, Sec. 8.1).  K is streamed to HBM once.  Both roles read the layers' brackets and coefficients 32 layers per
 // warp-wide load and find the segment starts with warp votes; the coefficients reach each
 // layer by shuffles.
 constexpr int kOT = kOpacityTile;                  // wavenumbers per unit
@@ -113,9 +114,9 @@ constexpr int kOCW = 4;                            // consumer warps
 constexpr int kOThreads = 32 * (kOCW + 1);         // + one producer warp
 static_assert(kOT == 64 * kOCW, "two wavenumbers per consumer lane");
 
-template <int MAXMOL, int MAXCIA, bool F16, bool EXPT>
-__global__ void __launch_bounds__(kOThreads, (EXPT && MAXMOL > 5) ? 2 : 3)
-k_opacity(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
+template <int MAXMOL, int MAXCIA, bool F16>
+__global__ void __launch_bounds__(kOThreads, MAXMOL > 5 ? 2 : 3)
+k_opacity_exp(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
           const __grid_constant__ CUtensorMap tm_cia, float* __restrict__ kbuf, long long kcols,
           int Bc, int n_tiles, int n_stages, int n_lb, int lb_size) {
   extern __shared__ unsigned char osm_raw[];
@@ -148,7 +149,6 @@ k_opacity(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
     float4 ha, hb;
     float2 ray;
     float xm[MAXMOL], yq[MAXCIA];
-    int zone;                                     // chemistry zone of ray, xm and yq
   };
   const int c2 = 2 * (warp * 32 + lane);             // column offset within the unit
   auto first_from = [&](long long u, CChunk& c) -> bool {
@@ -171,18 +171,15 @@ k_opacity(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
       c.hb = __ldg(op + 1);
     }
     if (unit_start) {
-      // the weights of the zone of the unit's first layer (zone 0 with constant mixing ratios)
-      // (the exponential scheme serves constant mixing ratios only: its register set is full)
-      c.zone = (!EXPT && p.buf.zoned) ? __shfl_sync(0xffffffffu, c.h.w, 0) : 0;
-      const int w = wbase + c.o.tile * kOT + c2;
-      c.ray = w < p.wn_pad ? rayleigh2(p, b, c.zone, w) : make_float2(0.f, 0.f);
-      item_weights<MAXMOL, MAXCIA>(p, b, c.zone, c.xm, c.yq);
+      const int w = wbase + c.o.tile * kOT + c2;        // constant mixing ratios: zone 0
+      c.ray = w < p.wn_pad ? rayleigh2(p, b, 0, w) : make_float2(0.f, 0.f);
+      item_weights<MAXMOL, MAXCIA>(p, b, 0, c.xm, c.yq);
     }
   };
   int seg = 0;
   int cip = -1, cit = -1, citc = -1, czone = -1;
-  float us[4][2] = {}, uc[2][2] = {};
-  // exponential T scheme: per molecule, P row and wavenumber log2 sigma at T_j and its step
+  float uc[2][2] = {};
+  // per molecule, P row and wavenumber log2 sigma at T_j and its step
   // to T_j+1 (or, for pairs marked in `lin`, the linear values)
   float lg[MAXMOL][2][2] = {}, dg[MAXMOL][2][2] = {};
   unsigned lin = 0u;
@@ -204,18 +201,18 @@ k_opacity(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
     const int N = cur.o.l_end, l0 = cur.l0;
     const int col = cur.o.tile * kOT + c2;
     const bool store = col < kcols, in_row = wbase + col < p.wn_pad;
-    float* dst = kbuf + ((size_t)cur.o.bc * p.max_layers + l0) * kcols + col;
+    float* dst = kbuf + k_index(cur.o.bc, col, l0, kcols, p.max_layers);
     if (l0 == cur.o.l_begin) cip = cit = citc = czone = -1;
-    const SegFlags f = segment_flags<!EXPT>(cur.h, l0, cur.o.l_begin, N, lane, has_mol, has_cia,
+    const SegFlags f = segment_flags<false>(cur.h, l0, cur.o.l_begin, N, lane, has_mol, has_cia,
                                             cip, cit, citc, czone);
     const float4 ha = cur.ha, hb = cur.hb;
-    float ray0 = cur.ray.x, ray1 = cur.ray.y;
+    const float ray0 = cur.ray.x, ray1 = cur.ray.y;
     const int n_here = min(32, N - l0);
     // K of one layer at this lane's two wavenumbers from the layer's coefficients, stored at dp
     auto one_layer = [&](float w0, float w1, float w2, float w3, float y0, float y1, float rho,
                          float kc, float* dp) {
       float k0 = fmaf(rho, ray0, kc), k1 = fmaf(rho, ray1, kc);
-      if constexpr (EXPT) {
+      {
         // w0, w1: rho x_max (1 - t_P), rho x_max t_P; w2: exponential T weight u; w3: linear
         // T weight t.  At each P row 2^(lg + u dg) = 2^64 x_m s1^(1-u) s2^u.
         float m0 = 0.f, m1 = 0.f;
@@ -250,75 +247,27 @@ k_opacity(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
           }
         }
         k0 = fmaf(m0, kExpScaleInv, k0); k1 = fmaf(m1, kExpScaleInv, k1);
-      } else {
-        k0 = fmaf(w0, us[0][0], k0); k1 = fmaf(w0, us[0][1], k1);
-        k0 = fmaf(w1, us[1][0], k0); k1 = fmaf(w1, us[1][1], k1);
-        k0 = fmaf(w2, us[2][0], k0); k1 = fmaf(w2, us[2][1], k1);
-        k0 = fmaf(w3, us[3][0], k0); k1 = fmaf(w3, us[3][1], k1);
       }
       k0 = fmaf(y0, uc[0][0], k0); k1 = fmaf(y0, uc[0][1], k1);
       k0 = fmaf(y1, uc[1][0], k0); k1 = fmaf(y1, uc[1][1], k1);
       if (store)
         __stcs(reinterpret_cast<float2*>(dp), in_row ? make_float2(k0, k1) : make_float2(0.f, 0.f));
     };
-    for (int i = 0; i < n_here;) {
+    // one layer per step (two per step would spill)
+    for (int i = 0; i < n_here; ++i) {
       if ((f.start >> i) & 1u) {                       // a new segment: take its stage
-        if (!EXPT && p.buf.zoned) {
-          // two-layer gases: a segment in another chemistry zone takes that zone's weights
-          const int zi = __shfl_sync(0xffffffffu, cur.h.w, i);
-          if (zi != cur.zone) {
-            const int b = p.b_off + cur.o.bc;
-            const int w = wbase + col;
-            cur.ray = in_row ? rayleigh2(p, b, zi, w) : make_float2(0.f, 0.f);
-            item_weights<MAXMOL, MAXCIA>(p, b, zi, cur.xm, cur.yq);
-            cur.zone = zi;
-            ray0 = cur.ray.x; ray1 = cur.ray.y;
-          }
-        }
-        bool ok;
-        if constexpr (EXPT)
-          ok = ring_consume_exp<kOT, MAXMOL, MAXCIA, F16>(p, rs, plan, ring, seg,
-                                                          (f.mol >> i) & 1u, (f.cia >> i) & 1u,
-                                                          c2, cur.xm, cur.yq, lg, dg, lin,
-                                                          anylin, uc, lane);
-        else
-          ok = ring_consume<kOT, 2, MAXMOL, MAXCIA, F16>(p, rs, plan, ring, seg,
-                                                         (f.mol >> i) & 1u, (f.cia >> i) & 1u,
-                                                         c2, cur.xm, cur.yq, us, uc, lane);
-        if (!ok) return;
+        if (!ring_consume_exp<kOT, MAXMOL, MAXCIA, F16>(p, rs, plan, ring, seg, (f.mol >> i) & 1u,
+                                                        (f.cia >> i) & 1u, c2, cur.xm, cur.yq, lg,
+                                                        dg, lin, anylin, uc, lane))
+          return;
         ++seg;
       }
-      // two layers of one segment at a time (their shuffles and FMA chains interleave); the
-      // exponential scheme keeps one layer per step (its register set would spill)
-      const bool pair = !EXPT && i + 1 < n_here && !((f.start >> (i + 1)) & 1u);
       const float a0 = __shfl_sync(0xffffffffu, ha.x, i), a1 = __shfl_sync(0xffffffffu, ha.y, i);
       const float a2 = __shfl_sync(0xffffffffu, ha.z, i), a3 = __shfl_sync(0xffffffffu, ha.w, i);
       const float b0 = __shfl_sync(0xffffffffu, hb.x, i), b1 = __shfl_sync(0xffffffffu, hb.y, i);
       const float b2 = __shfl_sync(0xffffffffu, hb.z, i), b3 = __shfl_sync(0xffffffffu, hb.w, i);
-      if (pair) {
-        const int j = i + 1;
-        const float e0 = __shfl_sync(0xffffffffu, ha.x, j), e1 = __shfl_sync(0xffffffffu, ha.y, j);
-        const float e2 = __shfl_sync(0xffffffffu, ha.z, j), e3 = __shfl_sync(0xffffffffu, ha.w, j);
-        const float f0 = __shfl_sync(0xffffffffu, hb.x, j), f1 = __shfl_sync(0xffffffffu, hb.y, j);
-        const float f2 = __shfl_sync(0xffffffffu, hb.z, j), f3 = __shfl_sync(0xffffffffu, hb.w, j);
-        one_layer(a0, a1, a2, a3, b0, b1, b2, b3, dst);
-        one_layer(e0, e1, e2, e3, f0, f1, f2, f3, dst + kcols);
-        dst += 2 * kcols;
-        i += 2;
-      } else {
-        one_layer(a0, a1, a2, a3, b0, b1, b2, b3, dst);
-        dst += kcols;
-        i += 1;
-      }
-    }
-    // the next chunk of the same unit continues with the zone weights this one ended with
-    if (!EXPT && p.buf.zoned && have_next && nxt.u == cur.u) {
-      nxt.ray = cur.ray;
-      nxt.zone = cur.zone;
-#pragma unroll
-      for (int m = 0; m < MAXMOL; ++m) nxt.xm[m] = cur.xm[m];
-#pragma unroll
-      for (int q = 0; q < MAXCIA; ++q) nxt.yq[q] = cur.yq[q];
+      one_layer(a0, a1, a2, a3, b0, b1, b2, b3, dst);
+      dst += kTW;
     }
     cur = nxt;
     have = have_next;
@@ -357,11 +306,11 @@ int sm_count() {
   return n;
 }
 
-template <int MAXMOL, int MAXCIA, bool F16, bool EXPT = false>
+template <int MAXMOL, int MAXCIA, bool F16>
 cudaError_t launch_opacity_t(const FwdParams& p, const CUtensorMap& sig, const CUtensorMap& cia,
                              int Bc, float* kbuf, long long kcols, int per_sm_cap,
                              cudaStream_t s) {
-  auto kern = k_opacity<MAXMOL, MAXCIA, F16, EXPT>;
+  auto kern = k_opacity_exp<MAXMOL, MAXCIA, F16>;
   // CTAs per SM: what the registers allow (at most 3, or the caller's cap), then the deepest
   // ring that fits them
   int per_sm = 0;
@@ -395,16 +344,6 @@ template <bool F16>
 cudaError_t launch_opacity_p(const FwdParams& p, const CUtensorMap& sig, const CUtensorMap& cia,
                              int Bc, float* kbuf, long long kcols, int cap, cudaStream_t s) {
   static_assert(TR_MAX_MOL == 8 && TR_MAX_CIA == 4, "opacity instantiations cover the limits");
-  if (p.interp_mode == TR_INTERP_EXP) {              // exponential T scheme (Sec. 5)
-    if (p.n_mol <= 2) return launch_opacity_t<2, 4, F16, true>(p, sig, cia, Bc, kbuf, kcols, cap, s);
-    if (p.n_mol <= 5) return launch_opacity_t<5, 4, F16, true>(p, sig, cia, Bc, kbuf, kcols, cap, s);
-    return launch_opacity_t<8, 4, F16, true>(p, sig, cia, Bc, kbuf, kcols, cap, s);
-  }
-  if (p.n_cia <= 2) {
-    if (p.n_mol <= 2) return launch_opacity_t<2, 2, F16>(p, sig, cia, Bc, kbuf, kcols, cap, s);
-    if (p.n_mol <= 5) return launch_opacity_t<5, 2, F16>(p, sig, cia, Bc, kbuf, kcols, cap, s);
-    return launch_opacity_t<8, 2, F16>(p, sig, cia, Bc, kbuf, kcols, cap, s);
-  }
   if (p.n_mol <= 2) return launch_opacity_t<2, 4, F16>(p, sig, cia, Bc, kbuf, kcols, cap, s);
   if (p.n_mol <= 5) return launch_opacity_t<5, 4, F16>(p, sig, cia, Bc, kbuf, kcols, cap, s);
   return launch_opacity_t<8, 4, F16>(p, sig, cia, Bc, kbuf, kcols, cap, s);
@@ -453,8 +392,8 @@ __device__ __forceinline__ bool wait_slot(const int* slot_unit, int k, const int
 
 template <int W>
 __global__ void __launch_bounds__(32 * (W + 1), 1)
-k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, long long kcols, int Bc,
-                int n_tiles, int n_slots) {
+k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int n_tiles,
+                int n_slots) {
   extern __shared__ unsigned char csm_raw[];
   __shared__ __align__(8) uint64_t kfull[kMaxSlots], kempty[kMaxSlots], dlfull;
   __shared__ int abort_flag, next_item, done[kMaxSlots], slot_unit[kMaxSlots];
@@ -522,7 +461,7 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, long long
       mbar_arrive_expect_tx(&kfull[sl], (uint32_t)nbox * kCB * kTW * 4);
       float* Kt = reinterpret_cast<float*>(base + sl * lay.slot);
       for (int i = 0; i < nbox; ++i)
-        tma_load_2d(Kt + (size_t)i * kCB * kTW, &tm_k, tile * kTW, bc * p.max_layers + i * kCB,
+        tma_load_2d(Kt + (size_t)i * kCB * kTW, &tm_k, 0, (bc * n_tiles + tile) * p.max_layers + i * kCB,
                     &kfull[sl]);
     }
     // every copy issued has landed before the CTA may exit
@@ -615,6 +554,24 @@ int forward_chunk_items(int B, int max_layers, int wn_begin, int wn_count) {
   return (int)std::min<size_t>((size_t)std::max(B, 1), n);
 }
 
+// All items and a slab of the wavenumbers where the buffer holds at least kMinCols of them, so a
+// slab's table rows are read once from HBM for all items (64 full-size atmospheres: 3 slabs
+// instead of 3 runs of items over the whole 2.4 GB of tables); else fewer items.  Buffers
+// smaller than 2 GiB, down to ones that stay in L2, were slower: every launch costs the opacity
+// and contraction kernels a last wave (64 atmospheres: 4.0 ms in 3 slabs, 5.0 ms in 20).
+KSplit forward_split(int B, int max_layers, int wn_begin, int wn_count) {
+  const long long cols = forward_kcols(wn_begin, wn_count);
+  const size_t budget = forward_kbuf_bytes(B, max_layers, wn_begin, wn_count);
+  constexpr long long kMinCols = 2048;
+  const long long fit = (long long)(budget / (sizeof(float) * (size_t)max_layers * std::max(B, 1)));
+  if (fit >= cols) return {std::max(B, 1), (int)cols};
+  const long long want = std::min(cols, std::max(fit / kTW * kTW, kMinCols));
+  const long long n = (cols + want - 1) / want;                    // slabs of about equal width
+  const long long c = ((cols + n - 1) / n + kTW - 1) / kTW * kTW;
+  const long long items = (long long)(budget / (sizeof(float) * (size_t)max_layers * c));
+  return {(int)std::max<long long>(1, std::min<long long>(items, B)), (int)c};
+}
+
 long long forward_kcols(int wn_begin, int wn_count) {
   const int w_first = wn_first(wn_begin);
   return (long long)((wn_begin + wn_count - w_first + kTW - 1) / kTW) * kTW;
@@ -627,19 +584,23 @@ size_t forward_kbuf_bytes(int B, int max_layers, int wn_begin, int wn_count) {
          max_layers * cols;
 }
 
-cudaError_t launch_opacity(const FwdParams& p, const CUtensorMap* tm_sig,
-                           const CUtensorMap* tm_cia, int Bc, float* kbuf, int per_sm_cap,
-                           cudaStream_t s) {
+cudaError_t launch_opacity(const FwdParams& p, const tr_tables* t, int Bc, float* kbuf,
+                           int per_sm_cap, cudaStream_t s) {
   if (Bc <= 0 || p.wn_count <= 0) return cudaSuccess;
   const long long kcols = (long long)n_tiles_of(p) * kTW;
-  return p.logsig16
-             ? launch_opacity_p<true>(p, *tm_sig, *tm_cia, Bc, kbuf, kcols, per_sm_cap, s)
-             : launch_opacity_p<false>(p, *tm_sig, *tm_cia, Bc, kbuf, kcols, per_sm_cap, s);
+  const bool f16 = p.logsig16 != nullptr;
+  if (p.interp_mode == TR_INTERP_LINEAR) {
+    const RowMaps tm{f16 ? &t->tm_row_t16 : &t->tm_row_t32, f16 ? &t->tm_row_p16 : &t->tm_row_p32,
+                     &t->tm_row_cia};
+    return launch_opacity_rows(p, tm, Bc, kbuf, kcols, per_sm_cap, s);
+  }
+  return f16 ? launch_opacity_p<true>(p, t->tm_sig16, t->tm_cia, Bc, kbuf, kcols, per_sm_cap, s)
+             : launch_opacity_p<false>(p, t->tm_sig32, t->tm_cia, Bc, kbuf, kcols, per_sm_cap, s);
 }
 
 template <int W>
-cudaError_t launch_contract_t(const FwdParams& p, const CUtensorMap& tm, long long kcols, int Bc,
-                              int tiles, int slots, uint32_t smem, cudaStream_t s) {
+cudaError_t launch_contract_t(const FwdParams& p, const CUtensorMap& tm, int Bc, int tiles,
+                              int slots, uint32_t smem, cudaStream_t s) {
   auto kern = k_contract_fp32<W>;
   cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (e != cudaSuccess) return e;
@@ -651,7 +612,7 @@ cudaError_t launch_contract_t(const FwdParams& p, const CUtensorMap& tm, long lo
   // the kernel counts units and (unit, ray tile) work items in 32 bits
   if (units * ((p.max_layers + kRT - 1) / kRT) > 0x7fffffffLL) return cudaErrorInvalidValue;
   const int grid = (int)std::min<long long>(units, (long long)sm_count());
-  kern<<<grid, 32 * (W + 1), smem, s>>>(p, tm, kcols, Bc, tiles, slots);
+  kern<<<grid, 32 * (W + 1), smem, s>>>(p, tm, Bc, tiles, slots);
   return cudaGetLastError();
 }
 
@@ -666,10 +627,8 @@ cudaError_t launch_contract_fp32(const FwdParams& p, int Bc, const float* kbuf, 
   kind = contract_kind(kind, p.max_layers);
   if (kind == kContractTC) return launch_contract_tc(p, Bc, kbuf, dl_tiles, s);
   const int tiles = n_tiles_of(p);
-  const long long kcols = (long long)tiles * kTW;
   CUtensorMap tm{};
-  if (!encode_2d_f32(&tm, kbuf, (unsigned long long)kcols,
-                     (unsigned long long)Bc * p.max_layers, (unsigned long long)kcols * 4, kTW,
+  if (!encode_2d_f32(&tm, kbuf, kTW, (unsigned long long)Bc * tiles * p.max_layers, kTW * 4, kTW,
                      kCB))
     return cudaErrorInvalidValue;
   constexpr uint32_t kSmemMax = 227u * 1024u;
@@ -680,8 +639,8 @@ cudaError_t launch_contract_fp32(const FwdParams& p, int Bc, const float* kbuf, 
   if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
   // eleven contraction warps (twelve plus the producer would be held to 128 registers and
   // spill; eleven keep 168), or eight
-  if (kind == kContractFfma11) return launch_contract_t<11>(p, tm, kcols, Bc, tiles, slots, smem, s);
-  return launch_contract_t<8>(p, tm, kcols, Bc, tiles, slots, smem, s);
+  if (kind == kContractFfma11) return launch_contract_t<11>(p, tm, Bc, tiles, slots, smem, s);
+  return launch_contract_t<8>(p, tm, Bc, tiles, slots, smem, s);
 }
 
 }  // namespace tr

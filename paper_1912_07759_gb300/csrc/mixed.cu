@@ -66,8 +66,7 @@ __global__ void k_dl_bf16(ItemBuffers buf, int max_layers, int NP, int KP,
 
 struct UmmaParams {
   FwdParams f;                     // item buffers, range, output, chunk offset
-  const float* kbuf;               // [chunk items][max_layers][kcols] FP32 K
-  long long kcols;
+  const float* kbuf;               // [chunk items][128-wn tiles][max_layers][128] FP32 K
   const __nv_bfloat16* dl16;       // [B][2][NP][KP]
   int NP, KP, tmem_cols;
 };
@@ -121,7 +120,7 @@ k_contract_umma(UmmaParams mp) {
   //      zero.  A thread packs 8 consecutive layers of one wavenumber (one 16-byte row of a
   //      core matrix) and stores it whole: consecutive threads fill consecutive rows, so the
   //      stores are free of bank conflicts.
-  const float* src = mp.kbuf + (size_t)blockIdx.y * p.max_layers * mp.kcols + (size_t)blockIdx.x * kMT;
+  const float* src = mp.kbuf + ((size_t)blockIdx.y * gridDim.x + blockIdx.x) * p.max_layers * kMT;
   for (int item = tid; item < kMT * (KP / 8); item += kMThreads) {
     const int v = item & (kMT - 1), lg = item / kMT;
     uint32_t hw[4], lw[4];
@@ -131,7 +130,7 @@ k_contract_umma(UmmaParams mp) {
 #pragma unroll
       for (int h = 0; h < 2; ++h) {
         const int l = lg * 8 + 2 * q + h;
-        x[h] = (l < N) ? __ldcs(src + (size_t)l * mp.kcols + v) : 0.f;
+        x[h] = (l < N) ? __ldcs(src + (size_t)l * kMT + v) : 0.f;
       }
       const __nv_bfloat162 hi2 = __floats2bfloat162_rn(x[0], x[1]);
       const float2 hf = __bfloat1622float2(hi2);
@@ -299,8 +298,8 @@ k_contract_umma_p(UmmaParams mp, const __grid_constant__ CUtensorMap tm_k, int B
         uint8_t* st = base + s * lay.stage;
         mbar_arrive_expect_tx(&sfull[s], lay.stage + (new_item ? dl_bytes : 0u));
         for (int i = 0; i < KP / 8; ++i)
-          tma_load_2d(st + (size_t)i * 8 * kMT * 4, &tm_k, tile * kMT,
-                      bc * p.max_layers + i * 8, &sfull[s]);
+          tma_load_2d(st + (size_t)i * 8 * kMT * 4, &tm_k, 0,
+                      (bc * n_tiles + tile) * p.max_layers + i * 8, &sfull[s]);
         if (new_item) {
           bulk_g2s(B_hi, mp.dl16 + (size_t)b * 2 * NP * KP, dl_bytes, &sfull[s]);
           dl_item = b;
@@ -482,15 +481,13 @@ cudaError_t launch_contract_umma(const FwdParams& p, int Bc, const float* kbuf, 
   const int w_first = wn_first(p.wn_begin);
   const int tiles = (p.wn_begin + p.wn_count - w_first + kMT - 1) / kMT;
   mp.kbuf = kbuf;
-  mp.kcols = (long long)tiles * kMT;
   mp.dl16 = static_cast<const __nv_bfloat16*>(dl16);
   mp.NP = NP; mp.KP = KP; mp.tmem_cols = tmem_cols_for(NP);
   if (KP <= kPMaxKP && UmmaPLayout(KP, NP).total <= 227u * 1024u) {
     // persistent warp-specialized form: one CTA per SM over a contiguous range of units
     CUtensorMap tm{};
-    if (!encode_2d_f32(&tm, kbuf, (unsigned long long)mp.kcols,
-                       (unsigned long long)Bc * p.max_layers, (unsigned long long)mp.kcols * 4,
-                       kMT, 8))
+    if (!encode_2d_f32(&tm, kbuf, kMT, (unsigned long long)Bc * tiles * p.max_layers, kMT * 4, kMT,
+                       8))
       return cudaErrorInvalidValue;
     const uint32_t smem = UmmaPLayout(KP, NP).total;
     cudaError_t e = cudaFuncSetAttribute(k_contract_umma_p,

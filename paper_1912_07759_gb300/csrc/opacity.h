@@ -1,5 +1,5 @@
-// opacity.h -- device pieces shared by the TMA-staged opacity kernels (the streaming two-stage
-// kernel in forward_fp32.cu and the fused forward kernel in fused.cu):
+// opacity.h -- device pieces of the opacity kernels with a producer warp (the exponential scheme's
+// two-stage kernel in forward_fp32.cu and the fused forward kernel in fused.cu):
 //   * the shared-memory ring of table-row stages and its producer warp, which walks the work
 //     units' layers as segments (maximal runs of layers with the same (P, T) cell and CIA
 //     temperature bracket) and issues one tiled TMA load per segment for the molecules' four

@@ -162,8 +162,8 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
         uint8_t* st = base + s * lay.stage;
         mbar_arrive_expect_tx(&sfull[s], lay.stage);
         for (int i = 0; i < KP / 8; ++i)
-          tma_load_2d(st + (size_t)i * 8 * kTM * 4, &tm_k, tile * kTM,
-                      bc * p.max_layers + i * 8, &sfull[s]);
+          tma_load_2d(st + (size_t)i * 8 * kTM * 4, &tm_k, 0,
+                      (bc * n_tiles + tile) * p.max_layers + i * 8, &sfull[s]);
       }
       for (int i = 0; i < 2 && i < k; ++i) {      // every copy issued has landed
         const int kl = k - 1 - i;
@@ -372,10 +372,9 @@ cudaError_t launch_contract_tc(const FwdParams& p, int Bc, const float* kbuf, co
   const int w_first = wn_first(p.wn_begin);
   if (!tiles) return cudaErrorInvalidValue;
   const int tiles_w = (p.wn_begin + p.wn_count - w_first + kTM - 1) / kTM;
-  const long long kcols = (long long)tiles_w * kTM;
   CUtensorMap tm{};
-  if (!encode_2d_f32(&tm, kbuf, (unsigned long long)kcols, (unsigned long long)Bc * p.max_layers,
-                     (unsigned long long)kcols * 4, kTM, 8))
+  if (!encode_2d_f32(&tm, kbuf, kTM, (unsigned long long)Bc * tiles_w * p.max_layers, kTM * 4, kTM,
+                     8))
     return cudaErrorInvalidValue;
   const uint32_t smem = TcLayout(KP, NP).total;
   void (*kern)(FwdParams, CUtensorMap, int, int, const float*) = nullptr;

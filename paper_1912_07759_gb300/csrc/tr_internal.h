@@ -27,6 +27,8 @@
 #include <vector>
 #include "../../include/transit.h"
 
+struct tr_tables;
+
 namespace tr {
 
 // SI constants.  CODATA-2018 G, k_B, m_u; R_J as the paper states it (Sec. 8.2).
@@ -198,6 +200,8 @@ __host__ __device__ inline int wn_first(int wn_begin) { return wn_begin & ~7; }
 // Wavenumbers per CTA of the TMA-staged opacity kernel (one per thread): the inner box size of
 // the tables' tensor maps.
 constexpr int kOpacityTile = 256;
+// Wavenumbers per warp of the linear scheme's opacity kernel.
+constexpr int kRowTile = 256;
 // Wavenumbers per work unit of the fused forward kernel (the inner box of its tensor maps).
 constexpr int kFusedTile = 128;
 
@@ -229,17 +233,33 @@ enum { TR_DEVERR_TIMEOUT = 1 };
 size_t forward_kbuf_bytes(int B, int max_layers, int wn_begin, int wn_count);
 // Columns of a K row in the buffer: the range [wn_first(wn_begin), wn_begin + wn_count) rounded
 // up to the contraction's 128-wavenumber tiles; K of chunk item c, layer l, column x is at
-// kbuf[(c * max_layers + l) * kcols + x].
+// kbuf[k_index(c, x, l, kcols, max_layers)].  The layout is tile-major: the 128 wavenumbers of a
+// contraction unit are one contiguous block [layers][128], so the opacity kernel writes and the
+// contraction reads whole blocks.
+constexpr int kKTile = 128;
+__host__ __device__ inline size_t k_index(int c, long long x, int l, long long kcols,
+                                          int max_layers) {
+  return (((size_t)c * (size_t)(kcols / kKTile) + (size_t)(x / kKTile)) * max_layers + l) * kKTile +
+         (size_t)(x % kKTile);
+}
 long long forward_kcols(int wn_begin, int wn_count);
 int forward_chunk_items(int B, int max_layers, int wn_begin, int wn_count);
+// How a two-stage forward of more items than the K buffer holds is cut: `items` items x `cols`
+// K columns at a time (the same buffer).
+struct KSplit { int items, cols; };
+KSplit forward_split(int B, int max_layers, int wn_begin, int wn_count);
 // Opacity of items [p.b_off, p.b_off + Bc): FP32 tables, or the FP16 log tables when
-// p.logsig16 is set (decoded on the fly).  tm_sig / tm_cia: tensor maps of the table in use
-// and of the CIA table (boxes {kOpacityTile, 2, 2, n_mol} and {kOpacityTile, 2, n_cia}).
+// p.logsig16 is set (decoded on the fly); t: the tables, for their tensor maps.
 // per_sm_cap: at most this many CTAs per SM (0: up to 3, as registers allow); the ring of
 // each takes the shared memory the others leave.
-cudaError_t launch_opacity(const FwdParams& p, const CUtensorMap* tm_sig,
-                           const CUtensorMap* tm_cia, int Bc, float* kbuf, int per_sm_cap,
-                           cudaStream_t s);
+cudaError_t launch_opacity(const FwdParams& p, const tr_tables* t, int Bc, float* kbuf,
+                           int per_sm_cap, cudaStream_t s);
+// The same with the linear temperature scheme (opacity_rows.cu), which launch_opacity takes.
+// Tensor maps with the inner box kRowTile wavenumbers: sigma boxes of two T rows at one P and of
+// two P rows at one T of every molecule, CIA boxes of one T row of every pair.
+struct RowMaps { const CUtensorMap *t_pair, *p_pair, *cia; };
+cudaError_t launch_opacity_rows(const FwdParams& p, const RowMaps& tm, int Bc, float* kbuf,
+                                long long kcols, int per_sm_cap, cudaStream_t s);
 // The FP32 path's contraction + depth for items [p.b_off, p.b_off + Bc) reading K.  `kind`:
 // kContractTC the 3xTF32 tensor-core kernel (tc_fp32.cu; layer counts up to 112),
 // kContractFfma8 / kContractFfma11 the FFMA kernel with eight or eleven contraction warps (one
@@ -465,6 +485,7 @@ struct tr_tables {
   CUtensorMap tm_sig32{};
   CUtensorMap tm_sig16{};
   CUtensorMap tm_cia{};
+  CUtensorMap tm_row_t32{}, tm_row_p32{}, tm_row_t16{}, tm_row_p16{}, tm_row_cia{};   // RowMaps
   CUtensorMap tm_sig32_f{};
   CUtensorMap tm_cia_f{};
   size_t device_bytes = 0;
