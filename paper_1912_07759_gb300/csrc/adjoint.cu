@@ -35,7 +35,8 @@ constexpr int kAT = 64;           // wavenumbers per adjoint CTA (2 per lane)
 constexpr int kAThreads = 256;
 constexpr int kAWarps = kAThreads / 32;
 constexpr int kRT = 8;            // rays (or layers) per register tile
-constexpr int kItemThreads = 128;
+constexpr int kItemThreads = 256;    // half over layers, half over radii
+constexpr int kItemHalf = kItemThreads / 2;
 
 // Float index of element (row, c) of the [rows][kAT] K and G_tau tiles: a row's 16-byte chunks
 // are XOR-swizzled by row / 4, so the G_DL blocks' float4 reads of rows 4 apart (one per
@@ -44,22 +45,32 @@ __device__ __forceinline__ int tix(int row, int c) {
   return row * kAT + ((((c >> 2) ^ (row >> 2)) & (kAT / 4 - 1)) << 2) + (c & 3);
 }
 
+// Jacobian rows done by one launch of each backward kernel: row r is bin first_bin + r, its tiles
+// are the slots [slot0[r], slot0[r + 1]).
+constexpr int kMaxRowSlots = 256;
+struct RowGroup {
+  int n_rows, first_bin;
+  uint16_t slot0[kMaxRowSlots + 1];
+  int tile[kMaxRowSlots];
+  uint8_t row[kMaxRowSlots];
+};
+
 struct AdjParams {
   FwdParams f;                    // tables and item buffers; wn_begin / wn_count = binned range
   const double* inv_dt;           // [n_t - 1]
   const double* inv_dtc;          // [n_t_cia - 1]
   const float* gd;                // [B][n_in] dL/dD at the native wavenumbers of the range
-  int n_in, tiles, n_feat;
+  int n_in, tiles, n_feat;        // tiles: slots per item of the partial sums
   float* part_a;                  // [B][tiles][npad]
   float* part_dl;                 // [B][tiles][npad][npad]  (ray j, shell l), j <= l
   float* part_f;                  // [B][tiles][max_layers][n_feat]
   float* part_rp;                 // [B][tiles]  sum_v G_D
   const float* kstore;            // the forward's K of the whole batch, or NULL: recompute
   long long kcols;                // columns of a K row in kstore
-  int tile0;                      // wavenumber tile of blockIdx.x == 0 (tiles = those launched)
-  // Jacobian row: >= 0 takes dL/dD from the bins' weights of this one bin (the row of
-  // dD_bin/dtheta), ignoring gd; -1 reads gd
-  int jac_bin;
+  // rows.n_rows == 0: one gradient, slot = wavenumber tile, dL/dD from gd.  Else a group of
+  // Jacobian rows: slot s takes tile rows.tile[s] of bin rows.bin[s], dL/dD from that bin's
+  // weights (its row of dD_bin/dtheta)
+  RowGroup rows;
   const int* t_ptr; const int* t_bin; const double* t_w;   // the bins' transpose (BinsDev)
 };
 
@@ -182,7 +193,10 @@ k_adjoint_tile(AdjParams a) {
   extern __shared__ __align__(16) float smem[];
   __shared__ __align__(8) uint64_t bar;
   const FwdParams& p = a.f;
-  const int b = blockIdx.y, tile = blockIdx.x;        // tile: index among the launched tiles
+  const int b = blockIdx.y, tile = blockIdx.x;        // tile: slot among the launched tiles
+  const bool jac = a.rows.n_rows > 0;
+  const int wtile = jac ? a.rows.tile[tile] : tile;   // wavenumber tile
+  const int jac_bin = jac ? a.rows.first_bin + a.rows.row[tile] : -1;
   const int N = p.buf.items[b].n_layers;
   if (N == 0) return;                                   // the item kernel zeroes its gradient
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -199,7 +213,7 @@ k_adjoint_tile(AdjParams a) {
   // that holds them
   float* red = (sp.red_in_kt() ? Kt : ray_s + (size_t)TR_MAX_SPECIES * kAT) +
                (size_t)warp * a.n_feat * kRedPitch;
-  const int w_first = wn_first(p.wn_begin) + (a.tile0 + tile) * kAT;
+  const int w_first = wn_first(p.wn_begin) + wtile * kAT;
 
   if (threadIdx.x == 0) { mbar_init(&bar, 1); mbar_fence_init(); }
   __syncthreads();
@@ -216,11 +230,11 @@ k_adjoint_tile(AdjParams a) {
     float g = 0.f;
     if (w >= p.wn_begin && w < p.wn_begin + a.n_in) {
       const int k = w - p.wn_begin;
-      if (a.jac_bin < 0) {
+      if (jac_bin < 0) {
         g = a.gd[(size_t)b * a.n_in + k];
       } else {                                          // dD_bin,jac_bin / dD at w
         for (int e = a.t_ptr[k]; e < a.t_ptr[k + 1]; ++e)
-          if (a.t_bin[e] == a.jac_bin) g = (float)a.t_w[e];
+          if (a.t_bin[e] == jac_bin) g = (float)a.t_w[e];
       }
     }
     gd_s[i] = g;
@@ -236,7 +250,7 @@ k_adjoint_tile(AdjParams a) {
   const bool in_row = w2 < p.wn_pad;
   const LayerDesc* LD = p.buf.layers + (size_t)b * p.max_layers;
   if constexpr (!RECOMP) {
-    const float* ks = a.kstore + k_index(b, (long long)(a.tile0 + tile) * kAT + 2 * lane, 0, a.kcols, p.max_layers);
+    const float* ks = a.kstore + k_index(b, (long long)wtile * kAT + 2 * lane, 0, a.kcols, p.max_layers);
     for (int l = warp; l < N; l += kAWarps)
       *reinterpret_cast<float2*>(Kt + tix(l, 2 * lane)) =
           __ldg(reinterpret_cast<const float2*>(ks + (size_t)l * kKTile));
@@ -570,31 +584,58 @@ k_adjoint_tile(AdjParams a) {
   }
 }
 
-// dL/dD at native wavenumbers of the binned range, and chi^2 (chi^2 mode) per item.
-__global__ void k_gd(BinsDev bd, int B, const double* __restrict__ binned,
-                     const double* __restrict__ obs, const double* __restrict__ sig,
-                     const double* __restrict__ gbin, const ItemGeom* __restrict__ items,
-                     double* __restrict__ chi2, float* __restrict__ gd, int n_in) {
+// dL/dD at native wavenumbers of the binned range (blockIdx.y: a run of kGdRun of them), and chi^2
+// (chi^2 mode) per item.  Latency-bound: the bins' terms are taken in parallel (one thread's
+// serial sum with a division per bin held the kernel at 33 us whatever the batch).
+constexpr int kGdThreads = 256, kGdRun = 2048;
+__global__ void __launch_bounds__(kGdThreads)
+k_gd(BinsDev bd, int B, const double* __restrict__ binned, const double* __restrict__ obs,
+     const double* __restrict__ sig, const double* __restrict__ gbin,
+     const ItemGeom* __restrict__ items, double* __restrict__ chi2, float* __restrict__ gd, int n_in) {
   __shared__ double gb[256];
-  const int b = blockIdx.x;
+  __shared__ double red[kGdThreads / 32];
+  const int b = blockIdx.x, t = threadIdx.x;
   const bool valid = items[b].status == TR_OK;
   const double* Db = binned + (size_t)b * bd.n_bin;
-  for (int k = threadIdx.x; k < bd.n_bin; k += blockDim.x) {
+  double c = 0.0;
+  if (t < bd.n_bin) {                                   // at most 256 bins
     double g = 0.0;
-    if (valid) g = gbin ? gbin[(size_t)b * bd.n_bin + k] : 2.0 * (Db[k] - obs[k]) / (sig[k] * sig[k]);
-    if (k < 256) gb[k] = g;
+    if (gbin) {
+      if (valid) g = gbin[(size_t)b * bd.n_bin + t];
+    } else {
+      const double d = Db[t] - obs[t], s = sig[t], r = d / s;
+      if (valid) g = 2.0 * d / (s * s);
+      c = r * r;
+    }
+    gb[t] = g;
   }
   __syncthreads();
-  if (threadIdx.x == 0 && chi2 && !gbin) {
-    double c = 0.0;
-    for (int k = 0; k < bd.n_bin; ++k) { const double r = (Db[k] - obs[k]) / sig[k]; c += r * r; }
-    chi2[b] = valid ? c : INFINITY;
-  }
-  for (int i = threadIdx.x; i < n_in; i += blockDim.x) {
+  const int i1 = min(n_in, (int)(blockIdx.y + 1) * kGdRun);
+  for (int i = blockIdx.y * kGdRun + t; i < i1; i += kGdThreads) {
     double g = 0.0;
     for (int e = bd.t_ptr[i]; e < bd.t_ptr[i + 1]; ++e) g += gb[bd.t_bin[e]] * bd.t_w[e];
     gd[(size_t)b * n_in + i] = (float)g;
   }
+  if (chi2 && !gbin && blockIdx.y == 0) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+    if ((t & 31) == 0) red[t >> 5] = c;
+    __syncthreads();
+    if (t == 0) {
+      for (int k = 1; k < (min(bd.n_bin, kGdThreads) + 31) / 32; ++k) c += red[k];
+      chi2[b] = valid ? c : INFINITY;
+    }
+  }
+}
+
+// gd of one Jacobian row: bin `bin`'s normalised weights.
+__global__ void k_row_gd(BinsDev bd, int bin, float* __restrict__ gd, int n_in) {
+  const int i = blockIdx.x * blockDim.x + threadIdx.x;
+  if (i >= n_in) return;
+  float g = 0.f;
+  for (int e = bd.t_ptr[i]; e < bd.t_ptr[i + 1]; ++e)
+    if (bd.t_bin[e] == bin) g = (float)bd.t_w[e];
+  gd[(size_t)blockIdx.y * n_in + i] = g;
 }
 
 // Sum of the wavenumber tiles' partial sums of one array [B][tiles][M] into its tile-0 slot,
@@ -609,8 +650,14 @@ struct TileSumArgs {
   float* arr[4];
   long long m[4];
   int tri[4];
+  int slots;                      // slots per item
+  RowGroup rows;                  // n_rows == 0: one row of all slots
 };
-__global__ void k_adjoint_sum(TileSumArgs ts, int B, int tiles) {
+__global__ void k_adjoint_sum(TileSumArgs ts, int B) {
+  const int r = blockIdx.z;
+  const int s0 = ts.rows.n_rows > 0 ? ts.rows.slot0[r] : 0;
+  const int tiles = (ts.rows.n_rows > 0 ? ts.rows.slot0[r + 1] : ts.slots) - s0;
+  if (tiles < 2) return;
   float* arr = ts.arr[blockIdx.y];
   const long long M = ts.m[blockIdx.y];
   const int tri = ts.tri[blockIdx.y];
@@ -619,7 +666,7 @@ __global__ void k_adjoint_sum(TileSumArgs ts, int B, int tiles) {
        i += (long long)gridDim.x * blockDim.x) {
     const long long b = i / M, m = i - b * M;
     if (tri > 0 && __all_sync(0xffffffffu, (int)m % tri < (int)m / tri)) continue;   // l < j
-    float* row = arr + (size_t)b * tiles * M + m;
+    float* row = arr + ((size_t)b * ts.slots + s0) * M + m;
     float s = row[0], c = 0.f;
     for (int t = 1; t < tiles; ++t) {
       const float y = __fsub_rn(row[(size_t)t * M], c);
@@ -635,31 +682,13 @@ struct ItemParams {
   GeomParams gp;
   const double* theta; int n_theta;
   ItemBuffers buf;
+  // partial sums [B][slots][...], each row's in its first slot (k_adjoint_sum)
   const float* part_a; const float* part_dl; const float* part_f; const float* part_rp;
-  int tiles, n_feat;              // partial sums are [B][tiles][...]
-  int n_sum;                      // tiles to add (1 after k_adjoint_sum)
-  double* grad;                   // item b's n_theta values at grad + b * grad_stride
-  long long grad_stride;
+  int slots, n_feat;
+  double* grad;                   // item b, row r: n_theta values at grad + b * item_stride + r * n_theta
+  long long item_stride;
+  RowGroup rows;                  // n_rows == 0: one row in slot 0
 };
-
-// Fixed-order tree sum over the CTA's threads of NV doubles per thread (red: [NV][threads]);
-// every thread gets the sums back in v.
-template <int NV>
-__device__ void block_sum_n(double (&v)[NV], double (*red)[kItemThreads]) {
-#pragma unroll
-  for (int i = 0; i < NV; ++i) red[i][threadIdx.x] = v[i];
-  __syncthreads();
-  for (int o = kItemThreads / 2; o > 0; o >>= 1) {
-    if (threadIdx.x < o) {
-#pragma unroll
-      for (int i = 0; i < NV; ++i) red[i][threadIdx.x] += red[i][threadIdx.x + o];
-    }
-    __syncthreads();
-  }
-#pragma unroll
-  for (int i = 0; i < NV; ++i) v[i] = red[i][0];
-  __syncthreads();
-}
 
 // (ah + al) - (bh + bl) to FP32 working precision (Knuth's TwoSum on the leading parts).
 __device__ __forceinline__ float diff_df(float ah, float al, float bh, float bl) {
@@ -669,80 +698,111 @@ __device__ __forceinline__ float diff_df(float ah, float al, float bh, float bl)
   return __fadd_rn(s, __fadd_rn(e, __fsub_rn(al, bl)));
 }
 
-// Dynamic shared memory of k_adjoint_item (bytes) for a maximum layer count.
-__host__ __device__ inline size_t item_smem_bytes(int NM) {
-  return sizeof(double) * (5 * (size_t)NM + 1)       // G_r, G_T, G_a, recursion factors, node weights
-         + sizeof(float2) * ((size_t)NM + 1)         // z as double-float
-         + sizeof(float) * ((size_t)NM + 1)          // r in FP32
-         + sizeof(int) * (size_t)NM + 16;            // node segment per layer
+// Values of the CTA sums: species, cloud top, d/dcz, d/dR_p, temperature nodes.
+constexpr int kItemRed = TR_MAX_SPECIES + 1 + 2 + TR_MAX_TNODES;
+
+// Dynamic shared memory of k_adjoint_item for a maximum layer count: FP64 per-layer arrays, the
+// CTA sums' terms, the altitudes and radii, the G_DL matrix (pitch npad + 1: its rows and columns
+// are both read without bank conflicts) and the features.
+struct ItemSmem {
+  int NM, npad, n_feat, n_val;
+  __host__ __device__ ItemSmem(int nm, int nf, int nv) : NM(nm), npad(pad8(nm)), n_feat(nf), n_val(nv) {}
+  __host__ __device__ size_t bytes() const {
+    return sizeof(double) * (5 * (size_t)NM + 1 + (size_t)n_val * kItemHalf) +
+           sizeof(float2) * ((size_t)NM + 1) +
+           sizeof(float) * ((size_t)NM + 1 + (size_t)npad * (npad + 1) + (size_t)NM * n_feat) +
+           sizeof(int) * (size_t)NM + 16;
+  }
+};
+
+// Adds t to the double-float sum (hi, lo): Knuth's TwoSum, the remainders collected in lo.
+__device__ __forceinline__ void add_df(float& hi, float& lo, float t) {
+  const float s = __fadd_rn(hi, t);
+  const float bb = __fsub_rn(s, hi);
+  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(t, bb)));
+  hi = s;
 }
 
-// One CTA per atmosphere.  GB300 runs FP64 at a small fraction of its FP32 rate, so the
-// O(N^2) path-length sensitivities are FP32 terms (from double-float altitudes, as the forward
-// path lengths) accumulated in FP64; per-layer and per-item work is spread over the threads;
-// the one serial chain left, the backward hydrostatic recursion, is one FP64 FMA per layer.
-constexpr int kItemRed = TR_MAX_SPECIES + 1 + 2 + TR_MAX_TNODES;   // values of the CTA sums
+// One CTA per (atmosphere, row).  GB300 runs FP64 at a small fraction of its FP32 rate and with
+// long latency (the SM completes one FP64 warp instruction per 19 cycles, a dependent one takes
+// about 140), so the kernel is bound by its FP64 instructions in large batches and by their
+// chains in small ones.  Four warps take the layers' terms in FP64 while the other four take the
+// O(N^2) path-length sensitivities, FP32 terms (from double-float altitudes, as the forward path
+// lengths) added into double-float sums without an FP64 instruction; the backward hydrostatic
+// recursion is a scan of its linear steps, and a warp adds each of the CTA's sums.  The G_DL
+// matrix and the features are staged in shared memory by coalesced reads (gathered from L2 by one
+// thread per radius they held the kernel at 112 us whatever the batch).  100 layers, 5 absorbers:
+// 8 atmospheres 114 -> 37 us, 1,024 193 -> 140 us, 50 rows of 128 atmospheres 5.58 -> 0.70 ms.
 __global__ void __launch_bounds__(kItemThreads)
 k_adjoint_item(ItemParams ip) {
   extern __shared__ double dsm[];
-  __shared__ double red[kItemRed][kItemThreads];
-  __shared__ double s_X[TR_MAX_SPECIES], s_GX[TR_MAX_SPECIES];
+  __shared__ double s_X[TR_MAX_SPECIES], s_sum[kItemRed];
   __shared__ double s_c[4];                            // cz, delta, mu, sum G_D
   const GeomParams& gp = ip.gp;
-  const int b = blockIdx.x, t = threadIdx.x;
+  const int b = blockIdx.x, t = threadIdx.x, warp = t >> 5, lane = t & 31;
+  const int row = blockIdx.y, slot = ip.rows.n_rows > 0 ? ip.rows.slot0[row] : 0;
   const int nth = ip.n_theta;
-  double* grad = ip.grad + (size_t)b * ip.grad_stride;
+  double* grad = ip.grad + (size_t)b * ip.item_stride + (size_t)row * nth;
   const ItemGeom ig = ip.buf.items[b];
   if (ig.status != TR_OK || ig.n_layers == 0) {
     for (int k = t; k < nth; k += kItemThreads) grad[k] = 0.0;
     return;
   }
-  const int N = ig.n_layers, NM = gp.max_layers, npad = ip.buf.npad;
+  const int N = ig.n_layers, NM = gp.max_layers, npad = ip.buf.npad, pitch = npad + 1;
   const double* th = ip.theta + (size_t)b * nth;
   const double* z = ip.buf.z + (size_t)b * (NM + 1);
   const double* T = ip.buf.tl + (size_t)b * NM;
   const LayerDesc* LD = ip.buf.layers + (size_t)b * NM;
+  const int nm = gp.n_mol, nq = gp.n_cia, ns = gp.n_species, ntn = gp.n_tnodes;
+  const int n_val = ns + 3 + ntn;                      // values of the CTA sums in use
   double* Gr = dsm;                 // [N + 1]
   double* GT = Gr + (NM + 1);       // [N]
   double* Ga = GT + NM;             // [N]
   double* fac = Ga + NM;            // [N] dr_{l+1} / dr_l of the recursion
   double* wn = fac + NM;            // [N] weight of node k_l + 1 in T_l
-  float2* zs = reinterpret_cast<float2*>(wn + NM);          // [N + 1]
-  float* rs = reinterpret_cast<float*>(zs + NM + 1);         // [N + 1]
-  int* kn = reinterpret_cast<int*>(rs + NM + 1);             // [N] node segment of layer l
+  double* val = wn + NM;            // [n_val][kItemHalf]
+  float2* zs = reinterpret_cast<float2*>(val + (size_t)n_val * kItemHalf);   // [N + 1]
+  float* rs = reinterpret_cast<float*>(zs + NM + 1);   // [N + 1]
+  float* G = rs + NM + 1;                              // [N][pitch] G_DL, zero beyond the diagonal
+  float* Fs = G + (size_t)npad * pitch;                // [N][n_feat]
+  int* kn = reinterpret_cast<int*>(Fs + (size_t)NM * ip.n_feat);   // [N] node segment of layer l
   const double rp = ig.r_p;
   const double inv_rs2 = gp.inv_rs2;
   const double ln10 = 2.302585092994046;
-  const int nm = gp.n_mol, nq = gp.n_cia, ntn = gp.n_tnodes;
+  const size_t ps = (size_t)b * ip.slots + slot;
 
-  // chemistry (as the profile kernel computes it), constants of the recursion
-  if (t < nm) s_X[t] = exp10(th[t]);
-  __syncthreads();
-  if (t == 0) {
+  // ---- staging; meanwhile warp 0 takes the chemistry (as the profile kernel computes it) and the
+  //      constants of the recursion
+  {
+    const float* g = ip.part_dl + ps * npad * npad;
+    for (int j = warp; j < N; j += kItemThreads / 32)
+      for (int l = lane; l < N; l += 32) G[j * pitch + l] = l >= j ? __ldg(g + (size_t)j * npad + l) : 0.f;
+    const float* f = ip.part_f + ps * NM * ip.n_feat;
+    for (int i = t; i < N * ip.n_feat; i += kItemThreads) Fs[i] = __ldg(f + i);
+    const float* pa = ip.part_a + ps * npad;
+    for (int j = t; j < N; j += kItemThreads) Ga[j] = (double)__ldg(pa + j);
+    for (int k = t; k <= N; k += kItemThreads) {
+      const double zk = z[k];
+      const float h = (float)zk;
+      zs[k] = make_float2(h, (float)(zk - (double)h));
+      rs[k] = (float)(rp + zk);
+    }
+  }
+  if (warp == 0) {
+    if (lane < nm) s_X[lane] = exp10(th[lane]);
+    __syncwarp();
     double sumx = 0.0, mu = 0.0;
     for (int m = 0; m < nm; ++m) { sumx += s_X[m]; mu = fma(s_X[m], gp.mass[m], mu); }
     const double rem = 1.0 - sumx;
-    for (int f = nm; f < gp.n_species; ++f) s_X[f] = gp.fill[f] * rem;
-    mu = fma(rem, gp.fill_mass, mu);
-    const double delta = (gp.ln_pmax - gp.ln_pmin) / N;
-    s_c[0] = (kKB * delta) / (mu * gp.amu_g_mp);
-    s_c[1] = delta;
-    s_c[2] = mu;
-    double grp = 0.0;
-    for (int q = 0; q < ip.n_sum; ++q) grp += ip.part_rp[(size_t)b * ip.tiles + q];
-    s_c[3] = grp;
-  }
-  // tile sums G_a; altitudes as double-float pairs and radii in FP32
-  for (int j = t; j < N; j += kItemThreads) {
-    double s = 0.0;
-    for (int q = 0; q < ip.n_sum; ++q) s += ip.part_a[((size_t)b * ip.tiles + q) * npad + j];
-    Ga[j] = s;
-  }
-  for (int k = t; k <= N; k += kItemThreads) {
-    const double zk = z[k];
-    const float h = (float)zk;
-    zs[k] = make_float2(h, (float)(zk - (double)h));
-    rs[k] = (float)(rp + zk);
+    if (lane >= nm && lane < ns) s_X[lane] = gp.fill[lane] * rem;
+    if (lane == 0) {
+      mu = fma(rem, gp.fill_mass, mu);
+      const double delta = (gp.ln_pmax - gp.ln_pmin) / N;
+      s_c[0] = (kKB * delta) / (mu * gp.amu_g_mp);
+      s_c[1] = delta;
+      s_c[2] = mu;
+      s_c[3] = (double)__ldg(ip.part_rp + ps);
+    }
   }
   __syncthreads();
   const double cz = s_c[0], delta = s_c[1], mu = s_c[2];
@@ -750,120 +810,134 @@ k_adjoint_item(ItemParams ip) {
   // ---- radii from path lengths and annulus weights
   //      DL[j][l] = 2 (s(l+1,j) - s(l,j)), s(k,j) = sqrt(r_k^2 - r_j^2):
   //      ds(k,j)/dr_k = r_k / s,  ds(k,j)/dr_j = -r_j / s;  r_k^2 - r_j^2 = (z_k - z_j)(r_k + r_j)
-  //      with z_k - z_j from the double-float altitudes; each term in FP32, sums in FP64
-  auto gdl = [&](int j, int l) -> float {    // sum over tiles of G_DL[j][l] (0 outside j<=l<N)
-    if (l < j || l >= N) return 0.f;
-    float s = 0.f;
-    for (int q = 0; q < ip.n_sum; ++q)
-      s += ip.part_dl[(((size_t)b * ip.tiles + q) * npad + j) * npad + l];
-    return s;
-  };
-  for (int k = t; k <= N; k += kItemThreads) {
-    const float2 zk = zs[k];
-    const float rk = rs[k];
-    double g = 0.0;
-    for (int j = 0; j < k; ++j) {                 // k as the outer radius of s(k, j)
-      const float gs = 2.f * (gdl(j, k - 1) - gdl(j, k));
-      if (gs != 0.f) {
+  //      with z_k - z_j from the double-float altitudes; each term in FP32, sums in double-float
+  const double dln = (gp.ln_pmin - gp.ln_pmax) / N;
+  const int f_dS = nm, f_R = 2 * nm, f_C = 2 * nm + ns, f_dC = f_C + nq, f_K = f_dC + nq;
+  double acc[TR_MAX_SPECIES + 3];                   // species, cloud top, d/dcz, d/dR_p
+#pragma unroll
+  for (int i = 0; i < TR_MAX_SPECIES + 3; ++i) acc[i] = 0.0;
+  if (t >= kItemHalf) {
+    for (int k = t - kItemHalf; k <= N; k += kItemHalf) {
+      const float2 zk = zs[k];
+      const float rk = rs[k];
+      float hi = 0.f, lo = 0.f;
+      float below = 0.f;                            // G[j][k]
+      for (int j = 0; j < k; ++j) {                 // k as the outer radius of s(k, j)
+        below = k < N ? G[j * pitch + k] : 0.f;
+        const float gs = 2.f * (G[j * pitch + k - 1] - below);
         const float2 zj = zs[j];
         const float s2 = diff_df(zk.x, zk.y, zj.x, zj.y) * (rk + rs[j]);
-        g += (double)(gs * rk * rsqrtf(s2));
+        add_df(hi, lo, gs != 0.f ? gs * rk * rsqrtf(s2) : 0.f);
       }
-    }
-    for (int kk = k + 1; kk <= N; ++kk) {         // k as the ray of s(kk, k)
-      const float gs = 2.f * (gdl(k, kk - 1) - gdl(k, kk));
-      if (gs != 0.f) {
+      float left = k < N ? G[k * pitch + k] : 0.f;  // G[k][kk - 1]
+      for (int kk = k + 1; kk <= N; ++kk) {         // k as the ray of s(kk, k)
+        const float right = kk < N ? G[k * pitch + kk] : 0.f;
+        const float gs = 2.f * (left - right);
+        left = right;
         const float2 zu = zs[kk];
         const float s2 = diff_df(zu.x, zu.y, zk.x, zk.y) * (rs[kk] + rk);
-        g -= (double)(gs * rk * rsqrtf(s2));
+        add_df(hi, lo, gs != 0.f ? -(gs * rk * rsqrtf(s2)) : 0.f);
       }
+      // a_j = (r_{j+1}^2 - r_j^2) / R_s^2
+      const double ga = ((k >= 1 ? Ga[k - 1] : 0.0) - (k < N ? Ga[k] : 0.0));
+      Gr[k] = fma(ga * 2.0 * (rp + z[k]), inv_rs2, (double)hi + (double)lo);
     }
-    // a_j = (r_{j+1}^2 - r_j^2) / R_s^2
-    const double rkd = rp + z[k];
-    if (k >= 1) g += Ga[k - 1] * 2.0 * rkd * inv_rs2;
-    if (k < N) g -= Ga[k] * 2.0 * rkd * inv_rs2;
-    Gr[k] = g;
-  }
-
-  // ---- per layer: opacity weights, densities, cloud; recursion factors; T-node weights
-  const double dln = (gp.ln_pmin - gp.ln_pmax) / N;
-  const int f_dS = nm, f_R = 2 * nm, f_C = 2 * nm + gp.n_species, f_dC = f_C + nq, f_K = f_dC + nq;
-  double acc[kItemRed];
+  } else {
+    // ---- per layer: opacity weights, densities, cloud; recursion factors; T-node weights
+    for (int l = t; l < N; l += kItemHalf) {
+      const LayerDesc& d = LD[l];
+      const float* F = Fs + l * ip.n_feat;
+      const double lnp0 = fma((double)l, dln, gp.ln_pmax), lnp1 = fma((double)(l + 1), dln, gp.ln_pmax);
+      const double lnp = 0.5 * (lnp0 + lnp1);
+      const double Tl = T[l], inv_t = 1.0 / Tl;
+      const double rho = (exp(lnp) * gp.inv_kb) * inv_t;
+      double gT = 0.0, grho = 0.0;
+      if (!(d.flags & kLayerMolZero)) {
+        double gt = 0.0;
 #pragma unroll
-  for (int i = 0; i < kItemRed; ++i) acc[i] = 0.0;
-  double* gx_loc = acc;                             // [TR_MAX_SPECIES]
-  double& glp = acc[TR_MAX_SPECIES];
-  for (int l = t; l < N; l += kItemThreads) {
-    double F[2 * TR_MAX_MOL + TR_MAX_SPECIES + 2 * TR_MAX_CIA + 1];
-    for (int f = 0; f < ip.n_feat; ++f) {
-      double s = 0.0;
-      for (int q = 0; q < ip.n_sum; ++q)
-        s += ip.part_f[(((size_t)b * ip.tiles + q) * NM + l) * ip.n_feat + f];
-      F[f] = s;
-    }
-    const LayerDesc& d = LD[l];
-    const double lnp0 = fma((double)l, dln, gp.ln_pmax), lnp1 = fma((double)(l + 1), dln, gp.ln_pmax);
-    const double lnp = 0.5 * (lnp0 + lnp1);
-    const double P = exp(lnp);
-    const double Tl = T[l];
-    const double rho = (P * gp.inv_kb) / Tl;
-    double gT = 0.0, grho = 0.0;
-    if (!(d.flags & kLayerMolZero)) {
-      for (int m = 0; m < nm; ++m) {
-        grho += F[m] * s_X[m];
-        gx_loc[m] += F[m] * rho;
-        gT += rho * s_X[m] * F[f_dS + m];
+        for (int m = 0; m < TR_MAX_MOL; ++m)
+          if (m < nm) {
+            const double f = F[m], x = s_X[m];
+            grho = fma(f, x, grho);
+            acc[m] = fma(f, rho, acc[m]);
+            gt = fma(x, (double)F[f_dS + m], gt);
+          }
+        gT = rho * gt;
       }
-    }
-    if (gp.has_ray) {
-      for (int s = 0; s < gp.n_species; ++s) {
-        const double R = F[f_R + s] * gp.ray_scale[s];
-        grho += R * s_X[s];
-        gx_loc[s] += R * rho;
+      if (gp.has_ray) {
+#pragma unroll
+        for (int s = 0; s < TR_MAX_SPECIES; ++s)
+          if (s < ns && F[f_R + s] != 0.f) {         // species without Rayleigh: exact zeros
+            const double R = F[f_R + s] * gp.ray_scale[s];
+            grho = fma(R, s_X[s], grho);
+            acc[s] = fma(R, rho, acc[s]);
+          }
       }
-    }
-    if (nq > 0 && !(d.flags & kLayerCiaZero)) {
-      for (int q = 0; q < nq; ++q) {
-        const double C = F[f_C + q] * gp.cia_scale[q], dC = F[f_dC + q] * gp.cia_scale[q];
-        const double xa = s_X[gp.cia_a[q]], xb = s_X[gp.cia_b[q]];
-        gT += rho * rho * xa * xb * dC;
-        grho += C * 2.0 * rho * xa * xb;
-        gx_loc[gp.cia_a[q]] += C * rho * rho * xb;
-        gx_loc[gp.cia_b[q]] += C * rho * rho * xa;
+      if (nq > 0 && !(d.flags & kLayerCiaZero)) {
+        for (int q = 0; q < nq; ++q) {
+          const double C = F[f_C + q] * gp.cia_scale[q], dC = F[f_dC + q] * gp.cia_scale[q];
+          const double xa = s_X[gp.cia_a[q]], xb = s_X[gp.cia_b[q]];
+          const double xx = rho * xa * xb, cr = C * rho * rho;
+          gT = fma(rho * xx, dC, gT);
+          grho = fma(C * 2.0, xx, grho);
+#pragma unroll
+          for (int s = 0; s < TR_MAX_SPECIES; ++s) {   // no indexed access to the sums
+            if (s == gp.cia_a[q]) acc[s] = fma(cr, xb, acc[s]);
+            if (s == gp.cia_b[q]) acc[s] = fma(cr, xa, acc[s]);
+          }
+        }
       }
-    }
-    gT += grho * (-rho / Tl);
-    if (gp.cloud_mode == TR_CLOUD_FRACTIONAL) {
-      // c_l = clamp((min(ln p_l, ln P_bot) - max(ln P_top, ln p_{l+1})) / Delta, 0, 1)
-      const double ln_top = th[nm + ntn + 1] * ln10;
-      const double hi = fmin(lnp0, gp.ln_cbot);
-      const double cf = (hi - fmax(ln_top, lnp1)) / delta;
-      if (cf > 0.0 && cf < 1.0 && ln_top > lnp1) glp += gp.kappa_cloud * F[f_K] * (-ln10 / delta);
-    }
-    GT[l] = gT;
-    // dr_{l+1}/dr_l: 1 + 2 cz T_l r_l (altitude-dependent gravity), 1 (constant)
-    fac[l] = gp.gravity_mode == TR_GRAV_CONST ? 1.0 : fma(2.0 * cz * Tl, rp + z[l], 1.0);
-    // temperature nodes: T_l linear in log10 P between nodes, clamped beyond them
-    int kseg = 0;
-    double f = 0.0;
-    if (ntn > 1) {
-      const double x = lnp * 0.43429448190325182765;
-      if (x >= gp.tnode_log10p[0]) { kseg = 0; f = 0.0; }
-      else if (x <= gp.tnode_log10p[ntn - 1]) { kseg = ntn - 2; f = 1.0; }
-      else {
-        while (!(gp.tnode_log10p[kseg] >= x && x >= gp.tnode_log10p[kseg + 1])) ++kseg;
-        f = (x - gp.tnode_log10p[kseg]) * gp.inv_dlog10p[kseg];
+      GT[l] = fma(-grho * rho, inv_t, gT);
+      if (gp.cloud_mode == TR_CLOUD_FRACTIONAL) {
+        // c_l = clamp((min(ln p_l, ln P_bot) - max(ln P_top, ln p_{l+1})) / Delta, 0, 1)
+        const double ln_top = th[nm + ntn + 1] * ln10;
+        const double hi = fmin(lnp0, gp.ln_cbot);
+        const double cf = hi - fmax(ln_top, lnp1);
+        if (cf > 0.0 && cf < delta && ln_top > lnp1)
+          acc[TR_MAX_SPECIES] += gp.kappa_cloud * F[f_K] * (-ln10 / delta);
       }
+      // dr_{l+1}/dr_l: 1 + 2 cz T_l r_l (altitude-dependent gravity), 1 (constant)
+      fac[l] = gp.gravity_mode == TR_GRAV_CONST ? 1.0 : fma(2.0 * cz * Tl, rp + z[l], 1.0);
+      // temperature nodes: T_l linear in log10 P between nodes, clamped beyond them
+      int kseg = 0;
+      double f = 0.0;
+      if (ntn > 1) {
+        const double x = lnp * 0.43429448190325182765;
+        if (x >= gp.tnode_log10p[0]) { kseg = 0; f = 0.0; }
+        else if (x <= gp.tnode_log10p[ntn - 1]) { kseg = ntn - 2; f = 1.0; }
+        else {
+          while (!(gp.tnode_log10p[kseg] >= x && x >= gp.tnode_log10p[kseg + 1])) ++kseg;
+          f = (x - gp.tnode_log10p[kseg]) * gp.inv_dlog10p[kseg];
+        }
+      }
+      kn[l] = kseg;
+      wn[l] = f;
     }
-    kn[l] = kseg;
-    wn[l] = f;
   }
   __syncthreads();
 
-  // ---- hydrostatic recursion, backwards (r_{l+1} = r_l + cz T_l r_l^2): one FMA per layer
-  if (t == 0) {
-    double g = Gr[N];
-    for (int l = N - 1; l >= 0; --l) {
+  // ---- hydrostatic recursion, backwards (r_{l+1} = r_l + cz T_l r_l^2): G_r of r_l is g_l = g_{l+1}
+  //      fac_l + Gr_l from g_N = Gr_N, a scan of linear maps g -> a g + c over the layers from the
+  //      top: each lane of warp 0 composes its run of layers, the lanes' maps are scanned, and the
+  //      run is replayed from the lane's entry value
+  if (warp == 0) {
+    const int per = (N + 31) / 32;
+    const int top = N - lane * per, bot = max(0, top - per);   // layers top - 1 .. bot
+    double a = 1.0, c = 0.0;
+    for (int l = top - 1; l >= bot; --l) {
+      a *= fac[l];
+      c = fma(c, fac[l], Gr[l]);
+    }
+#pragma unroll
+    for (int o = 1; o < 32; o <<= 1) {              // maps of lanes 0 .. lane, in that order
+      const double pa = __shfl_up_sync(0xffffffffu, a, o), pc = __shfl_up_sync(0xffffffffu, c, o);
+      if (lane >= o) { c = fma(pc, a, c); a *= pa; }
+    }
+    const double gN = Gr[N];
+    double g = fma(gN, a, c);                       // g at this lane's lowest radius
+    g = __shfl_up_sync(0xffffffffu, g, 1);
+    if (lane == 0) g = gN;
+    for (int l = top - 1; l >= bot; --l) {
       g = fma(g, fac[l], Gr[l]);
       Gr[l] = g;
     }
@@ -871,38 +945,60 @@ k_adjoint_item(ItemParams ip) {
   __syncthreads();
   // per layer, with G_r of r_{l+1}: dT_l and dcz (and, for constant gravity, dR_p) terms;
   // then the CTA sums of the mixing-ratio, cloud, cz, R_p and node terms
-  for (int l = t; l < N; l += kItemThreads) {
-    const double g1 = Gr[l + 1];
-    const double rl = gp.gravity_mode == TR_GRAV_CONST ? rp : rp + z[l];
-    const double gT = GT[l] + g1 * cz * rl * rl;
-    acc[TR_MAX_SPECIES + 1] += g1 * T[l] * rl * rl;                    // d/dcz
-    if (gp.gravity_mode == TR_GRAV_CONST)
-      acc[TR_MAX_SPECIES + 2] += g1 * 2.0 * cz * T[l] * rp;            // d/dR_p, direct
-    double* gnode = acc + TR_MAX_SPECIES + 3;
-    if (ntn == 1) {
-      gnode[0] += gT;
-    } else {
-      gnode[kn[l]] += gT * (1.0 - wn[l]);
-      gnode[kn[l] + 1] += gT * wn[l];
+  if (t < kItemHalf) {
+    double gnode[TR_MAX_TNODES];
+#pragma unroll
+    for (int k = 0; k < TR_MAX_TNODES; ++k) gnode[k] = 0.0;
+    for (int l = t; l < N; l += kItemHalf) {
+      const double g1 = Gr[l + 1];
+      const double rl = gp.gravity_mode == TR_GRAV_CONST ? rp : rp + z[l];
+      const double gr2 = g1 * rl * rl, Tl = T[l];
+      const double gT = fma(gr2, cz, GT[l]);
+      acc[TR_MAX_SPECIES + 1] = fma(gr2, Tl, acc[TR_MAX_SPECIES + 1]);   // d/dcz
+      if (gp.gravity_mode == TR_GRAV_CONST)
+        acc[TR_MAX_SPECIES + 2] += g1 * 2.0 * cz * Tl * rp;            // d/dR_p, direct
+      if (ntn == 1) {
+        gnode[0] += gT;
+      } else {
+        const double hi = gT * wn[l], lo = gT - hi;
+        const int k0 = kn[l];
+#pragma unroll
+        for (int k = 0; k < TR_MAX_TNODES; ++k) {
+          if (k == k0) gnode[k] += lo;
+          if (k == k0 + 1) gnode[k] += hi;
+        }
+      }
     }
+#pragma unroll
+    for (int s = 0; s < TR_MAX_SPECIES; ++s) if (s < ns) val[s * kItemHalf + t] = acc[s];
+#pragma unroll
+    for (int k = 0; k < 3; ++k) val[(ns + k) * kItemHalf + t] = acc[TR_MAX_SPECIES + k];
+#pragma unroll
+    for (int k = 0; k < TR_MAX_TNODES; ++k) if (k < ntn) val[(ns + 3 + k) * kItemHalf + t] = gnode[k];
   }
-  block_sum_n<kItemRed>(acc, red);
-  if (t == 0) {
-    for (int s = 0; s < gp.n_species; ++s) s_GX[s] = acc[s];
-    const double glp_sum = acc[TR_MAX_SPECIES], gcz = acc[TR_MAX_SPECIES + 1];
-    const double grp_dir = acc[TR_MAX_SPECIES + 2];
-    const double g_rp = Gr[0] + grp_dir + s_c[3] * 2.0 * rp * inv_rs2;
+  __syncthreads();
+  for (int v = warp; v < n_val; v += kItemThreads / 32) {
+    double s = 0.0;
+#pragma unroll
+    for (int k = 0; k < kItemHalf / 32; ++k) s += val[v * kItemHalf + 32 * k + lane];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+    if (lane == 0) s_sum[v] = s;
+  }
+  __syncthreads();
+  if (warp == 0) {
+    const double glp_sum = s_sum[ns], gcz = s_sum[ns + 1], grp_dir = s_sum[ns + 2];
     const double gmu = gcz * (-cz / mu);
     // chemistry: X_m = 10^theta_m, fill gases f (1 - sum X), mu = sum X_s m_s
     double sum_fill = 0.0;
-    for (int f = nm; f < gp.n_species; ++f) sum_fill += gp.fill[f] * (s_GX[f] + gmu * gp.mass[f]);
-    for (int m = 0; m < nm; ++m) {
-      const double gxm = s_GX[m] + gmu * gp.mass[m] - sum_fill;
-      grad[m] = gxm * s_X[m] * ln10;
+    for (int f = nm; f < ns; ++f) sum_fill += gp.fill[f] * (s_sum[f] + gmu * gp.mass[f]);
+    if (lane < nm) grad[lane] = (s_sum[lane] + gmu * gp.mass[lane] - sum_fill) * s_X[lane] * ln10;
+    if (lane < ntn) grad[nm + lane] = s_sum[ns + 3 + lane];
+    if (lane == 0) {
+      const double g_rp = Gr[0] + grp_dir + s_c[3] * 2.0 * rp * inv_rs2;
+      grad[nm + ntn] = g_rp * kRJup;
+      grad[nm + ntn + 1] = glp_sum;
     }
-    for (int k = 0; k < ntn; ++k) grad[nm + k] = acc[TR_MAX_SPECIES + 3 + k];
-    grad[nm + ntn] = g_rp * kRJup;
-    grad[nm + ntn + 1] = glp_sum;
   }
 }
 
@@ -1010,8 +1106,9 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
   if (d_grad) {
     KernelTimer kt(ctx, "k_gd", s);
-    k_gd<<<B, 256, 0, s>>>(bins->dev, B, binned, d_obs, d_sigma_obs, d_gbin, buf.items,
-                           d_gbin ? nullptr : d_chi2, gd, n_in);
+    k_gd<<<dim3(B, (n_in + kGdRun - 1) / kGdRun), kGdThreads, 0, s>>>(
+        bins->dev, B, binned, d_obs, d_sigma_obs, d_gbin, buf.items, d_gbin ? nullptr : d_chi2, gd,
+        n_in);
     err = cudaGetLastError();
   }
   if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
@@ -1049,59 +1146,91 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   itp.gp = batch_geom_params(t, d); itp.theta = d_theta; itp.n_theta = nth; itp.buf = buf;
   itp.part_a = part_a; itp.part_dl = part_dl; itp.part_f = part_f; itp.part_rp = part_rp;
   itp.n_feat = n_feat;
-  itp.n_sum = 1;                                            // tile 0 holds the sums
-  const size_t smem_i = item_smem_bytes(d->max_layers);
+  const size_t smem_i = ItemSmem(d->max_layers, n_feat, t->n_species + 3 + d->n_tnodes).bytes();
+  err = cudaFuncSetAttribute(k_adjoint_item, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_i);
+  if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint item kernel: ") + cudaGetErrorString(err));
 
-  // One backward pass over wavenumber tiles [tile0, tile0 + nt): the tile kernel's partial
-  // sums, their GPU-wide sum into tile 0, and the per-atmosphere kernel writing item b's
-  // gradient at grad + b * stride.  jac_bin < 0 takes dL/dD from gd, else the weights of bin
-  // jac_bin (one row of the Jacobian).
-  auto backward = [&](int jac_bin, int tile0, int nt, double* grad, long long stride) -> int {
-    ap.tile0 = tile0; ap.tiles = nt; ap.jac_bin = jac_bin;
+  // One backward pass over `slots` wavenumber tiles per item: the tile kernel's partial sums,
+  // their GPU-wide sum into each row's first slot, and the per-atmosphere kernel writing item b's
+  // row r at grad + b * stride + r * nth.  No rows: one gradient with dL/dD from gd.
+  auto backward = [&](const RowGroup& rows, int slots, double* grad, long long stride) -> int {
+    const int n_rows = std::max(rows.n_rows, 1);
+    ap.rows = rows; ap.tiles = slots;
     {
       KernelTimer kt(ctx, "k_adjoint_tile", s);
-      kern<<<dim3(nt, B), kAThreads, smem, s>>>(ap);
+      kern<<<dim3(slots, B), kAThreads, smem, s>>>(ap);
       err = cudaGetLastError();
     }
     if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint tile kernel: ") + cudaGetErrorString(err));
-    if (nt > 1) {
-      // the tiles' partial sums into tile 0 by a GPU-wide pass, so the per-atmosphere kernel
-      // reads one set of sums
+    if (slots > n_rows) {
+      // the tiles' partial sums into the rows' first slots by a GPU-wide pass, so the
+      // per-atmosphere kernel reads one set of sums
       KernelTimer kt(ctx, "k_adjoint_sum", s);
       TileSumArgs ts{};
       ts.arr[0] = part_a;  ts.m[0] = npad;
       ts.arr[1] = part_dl; ts.m[1] = (long long)npad * npad; ts.tri[1] = npad;
       ts.arr[2] = part_f;  ts.m[2] = (long long)d->max_layers * n_feat;
       ts.arr[3] = part_rp; ts.m[3] = 1;
+      ts.slots = slots; ts.rows = rows;
       const long long most = (long long)B * npad * npad;
       const int gx = (int)std::max<long long>(1, std::min<long long>((most + 255) / 256, 8LL * n_sm));
-      k_adjoint_sum<<<dim3(gx, 4), 256, 0, s>>>(ts, B, nt);
+      k_adjoint_sum<<<dim3(gx, 4, n_rows), 256, 0, s>>>(ts, B);
       err = cudaGetLastError();
       if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint sum kernel: ") + cudaGetErrorString(err));
     }
-    itp.tiles = nt; itp.grad = grad; itp.grad_stride = stride;
+    itp.rows = rows; itp.slots = slots; itp.grad = grad; itp.item_stride = stride;
     {
       KernelTimer kt(ctx, "k_adjoint_item", s);
-      k_adjoint_item<<<B, kItemThreads, smem_i, s>>>(itp);
+      k_adjoint_item<<<dim3(B, n_rows), kItemThreads, smem_i, s>>>(itp);
       err = cudaGetLastError();
     }
     if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint item kernel: ") + cudaGetErrorString(err));
     return TR_OK;
   };
   if (d_grad) {
-    rc = backward(-1, 0, tiles, d_grad, nth);
+    RowGroup one;
+    one.n_rows = 0; one.first_bin = 0;
+    rc = backward(one, tiles, d_grad, nth);
     if (rc != TR_OK) return rc;
   }
   if (d_jac) {
     // row k of dD_bin/dtheta: dL/dD is bin k's normalised weights, which vanish outside the
-    // bin's native range, so the pass covers only the tiles of that range
+    // bin's native range, so a row covers only the tiles of that range.  The rows go in groups
+    // of as many as the partial sums' space for one gradient (`tiles` slots per item) holds, one
+    // launch of each kernel per group: a launch per row left the GPU with one row's CTAs (128
+    // atmospheres, 50 bins of about 19 wavenumbers: 7.86 ms a call, in groups 2.3 ms).
     const int base = wn_first(bins->dev.i0);
     const int n_bin = bins->dev.n_bin;
-    for (int k = 0; k < n_bin; ++k) {
-      const int t0 = (bins->bin_lo[k] - base) / kAT;
-      const int t1 = (bins->bin_hi[k] - 1 - base) / kAT + 1;
-      rc = backward(k, t0, t1 - t0, d_jac + (size_t)k * nth, (long long)n_bin * nth);
+    const int cap = std::min(tiles, kMaxRowSlots);
+    auto first_tile = [&](int k) { return (bins->bin_lo[k] - base) / kAT; };
+    auto n_tiles = [&](int k) { return (bins->bin_hi[k] - 1 - base) / kAT + 1 - first_tile(k); };
+    for (int k0 = 0; k0 < n_bin;) {
+      RowGroup g;
+      g.n_rows = 0; g.first_bin = k0;
+      int slots = 0, k = k0;
+      for (; k < n_bin && slots + n_tiles(k) <= cap; ++k) {
+        g.slot0[g.n_rows] = (uint16_t)slots;
+        for (int q = 0; q < n_tiles(k); ++q, ++slots) {
+          g.tile[slots] = first_tile(k) + q;
+          g.row[slots] = (uint8_t)g.n_rows;
+        }
+        ++g.n_rows;
+      }
+      if (g.n_rows == 0) {
+        // a bin of more tiles than a group can list: its tiles one gradient-like pass, dL/dD
+        // written to gd
+        k_row_gd<<<dim3((n_in + 255) / 256, B), 256, 0, s>>>(bins->dev, k, gd, n_in);
+        err = cudaGetLastError();
+        if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
+        rc = backward(g, tiles, d_jac + (size_t)k * nth, (long long)n_bin * nth);
+        if (rc != TR_OK) return rc;
+        k0 = k + 1;
+        continue;
+      }
+      g.slot0[g.n_rows] = (uint16_t)slots;
+      rc = backward(g, slots, d_jac + (size_t)k0 * nth, (long long)n_bin * nth);
       if (rc != TR_OK) return rc;
+      k0 = k;
     }
   }
   return TR_OK;
