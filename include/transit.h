@@ -379,9 +379,8 @@ int tr_unpin_forward_config(tr_ctx* ctx, const tr_tables* tables, const tr_batch
 /*
  * Batched forward model plus hand-written adjoint (reverse-mode derivative of the same
  * discrete model; the paper has no gradient path: this serves gradient-based samplers and
- * Fisher matrices).  The backward passes reuse the forward's opacity K from the workspace
- * when its K buffer (2 GiB) holds the whole batch and recompute K from the tables when the
- * batch outgrows it.  Outputs, each written when its pointer is not NULL (at least one of
+ * Fisher matrices).  The backward passes reuse the forward's opacity K from the workspace; a
+ * batch that outgrows its K buffer (2 GiB) is taken in runs of items that fit it.  Outputs, each written when its pointer is not NULL (at least one of
  * d_grad, d_jac):
  *   d_grad[B][n_theta], in one of two modes:
  *     d_gbin != NULL: vector-Jacobian product.  d_gbin[B][n_bin] is an upstream gradient
@@ -398,9 +397,8 @@ int tr_unpin_forward_config(tr_ctx* ctx, const tr_tables* tables, const tr_batch
  * Invalid items get zero gradients and Jacobians (and chi^2 = +inf in chi^2 mode).  When
  * neither chi^2 nor d_binned is asked for, the forward runs only its geometry and opacity
  * stages (the backward passes need K, not the spectrum).
- *   recompute_k: 1 recomputes K in the backward pass; 0 or -1 (automatic) reuse the forward's
- *     K when the workspace's K buffer holds the whole batch (recomputing it otherwise).  The
- *     recomputation repeats the forward's arithmetic (the same sums in the same order), so
+ *   recompute_k: 1 recomputes K in the backward pass; 0 or -1 (automatic) reuse the forward's.
+ *     The recomputation repeats the forward's arithmetic (the same sums in the same order), so
  *     the choice changes the time, not the results (the GPU tests check bitwise equal
  *     gradients with FP32 tables).
  *   d_workspace: >= tr_batch_workspace_size(..., with_adjoint=1) bytes, or NULL.

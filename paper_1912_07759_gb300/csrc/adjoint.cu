@@ -12,9 +12,9 @@
 //   G_K_l(v)  = sum_{j<=l} DL[j][l] G_tau_j(v);  G_DL[j][l] = sum_v G_tau_j(v) K_l(v)
 //   per layer: sum_v G_K sigma_m, sum_v G_K dsigma_m/dT, sum_v G_K sigma_R,s, CIA alike,
 //              sum_v G_K                                          (k_adjoint_tile, FP32:
-//              K is the forward's, read back from the workspace's K buffer when that holds
-//              the whole batch, and recomputed from the tables when the batch outgrows it,
-//              with the opacity kernel's per-cell sums and per-layer FMAs, so bit for bit; tau
+//              K is the forward's, read back from the workspace's K buffer, the batch taken in
+//              runs of items that fit it; or, when asked for, recomputed from the tables with
+//              the opacity kernel's per-cell sums and per-layer FMAs, so bit for bit; tau
 //              is recomputed; with mixed precision the cross-sections come from the FP16
 //              log10 tables, decoded on the fly, and the forward runs the mixed path)
 //   then, per atmosphere (FP64 sums; the path-length terms in FP32 from double-float
@@ -65,7 +65,7 @@ struct AdjParams {
   float* part_dl;                 // [B][tiles][npad][npad]  (ray j, shell l), j <= l
   float* part_f;                  // [B][tiles][max_layers][n_feat]
   float* part_rp;                 // [B][tiles]  sum_v G_D
-  const float* kstore;            // the forward's K of the whole batch, or NULL: recompute
+  const float* kstore;            // the forward's K of the items, or NULL: recompute
   long long kcols;                // columns of a K row in kstore
   // rows.n_rows == 0: one gradient, slot = wavenumber tile, dL/dD from gd.  Else a group of
   // Jacobian rows: slot s takes tile rows.tile[s] of bin rows.bin[s], dL/dD from that bin's
@@ -245,7 +245,7 @@ k_adjoint_tile(AdjParams a) {
       ray_s[i] = w < p.wn_pad ? __ldg(p.ray + (size_t)sp2 * p.wn_pad + w) : 0.f;
     }
   }
-  // ---- K tile: the forward's, when its buffer holds the whole batch; else recomputed
+  // ---- K tile: the forward's, or recomputed
   const int w2 = w_first + 2 * lane;
   const bool in_row = w2 < p.wn_pad;
   const LayerDesc* LD = p.buf.layers + (size_t)b * p.max_layers;
@@ -1070,22 +1070,21 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   float* kbuf = reinterpret_cast<float*>(extra);
   void* dl16 = db > 0 ? extra + kb : nullptr;
   extra += kb + db;
-  const bool k_whole = forward_chunk_items(B, d->max_layers, bins->dev.i0, n_in) >= B;
-  const bool use_kstore = k_whole && recompute_k != 1;
-  // forward, in the two-stage form (the configuration tuned for this shape's forward, if
-  // any), which leaves K in kbuf; when one chunk holds the whole batch the backward passes
-  // read it back instead of recomputing it.  The binned spectrum is needed only for chi^2 or
-  // when asked for: otherwise (vector-Jacobian products, Jacobian) only the opacity stage
-  // runs, and not even that when the backward recomputes K.
+  // The batch in runs of as many items as the K buffer holds (equal runs): the forward, in the
+  // two-stage form (the configuration tuned for this shape's forward, if any), leaves their K in
+  // kbuf and the backward passes read it.  recompute_k == 1: the whole batch at once, K formed
+  // again from the tables by the tile kernel.  (Recomputing K where the batch outgrows the
+  // buffer, which this replaces, cost 65 us a tile against 50: 320 atmospheres of 18,905
+  // wavenumbers and 100 layers took 23.2 ms, in two runs 18.2.)  The binned spectrum is needed
+  // only for chi^2 or when asked for: otherwise (vector-Jacobian products, Jacobian) only the
+  // opacity stage runs, and not even that when the backward recomputes K.
+  const bool use_kstore = recompute_k != 1;
   const bool need_binned = chi2_mode || d_binned;
+  const int fit = use_kstore ? forward_chunk_items(B, d->max_layers, bins->dev.i0, n_in) : B;
+  const int n_runs = (B + fit - 1) / fit, run = (B + n_runs - 1) / n_runs;
   const auto it = ctx->tuned.find(batch_shape_key(t, d, B, bins, false, precision));
   ForwardChoice fc = it != ctx->tuned.end() ? it->second : ForwardChoice{kFormTwoStage, 0, 0, 0};
   fc.form = kFormTwoStage;
-  if (need_binned || use_kstore) {
-    rc = run_forward(ctx, t, d->max_layers, buf, B, bins->dev.i0, n_in, depth, n_in, precision,
-                     s, kbuf, dl16, &fc, /*opacity_only=*/!need_binned);
-    if (rc != TR_OK) return rc;
-  }
   const int tiles = (bins->dev.i1 - wn_first(bins->dev.i0) + kAT - 1) / kAT;
   const int npad = pad8(d->max_layers);
   const int n_feat = 2 * t->n_mol + t->n_species + 2 * t->n_cia + 1;
@@ -1099,24 +1098,11 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   float* part_rp = reinterpret_cast<float*>(e); e += al(sizeof(float) * (size_t)B * tiles);
   double* binned = d_binned ? d_binned : reinterpret_cast<double*>(e);
   cudaError_t err = cudaSuccess;
-  if (need_binned) {
-    KernelTimer kt(ctx, "k_bin", s);
-    err = launch_bin(bins->dev, B, depth, n_in, bins->dev.i0, binned, s);
-  }
-  if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
-  if (d_grad) {
-    KernelTimer kt(ctx, "k_gd", s);
-    k_gd<<<dim3(B, (n_in + kGdRun - 1) / kGdRun), kGdThreads, 0, s>>>(
-        bins->dev, B, binned, d_obs, d_sigma_obs, d_gbin, buf.items, d_gbin ? nullptr : d_chi2, gd,
-        n_in);
-    err = cudaGetLastError();
-  }
-  if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
   AdjParams ap{};
   ap.f.sigma = t->d_sigma; ap.f.n_mol = t->n_mol; ap.f.n_p = t->n_p; ap.f.n_t = t->n_t;
   ap.f.wn_pad = t->wn_pad; ap.f.cia = t->d_cia; ap.f.n_cia = t->n_cia; ap.f.n_t_cia = t->n_t_cia;
   ap.f.ray = t->has_ray ? t->d_ray : nullptr; ap.f.n_species = t->n_species;
-  ap.f.max_layers = d->max_layers; ap.f.buf = buf; ap.f.wn_begin = bins->dev.i0;
+  ap.f.max_layers = d->max_layers; ap.f.wn_begin = bins->dev.i0;
   ap.f.wn_count = n_in; ap.f.dev_err = ctx->dev_err;
   if (mixed) {
     ap.f.logsig16 = t->d_logsig16;
@@ -1143,7 +1129,7 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   ItemParams itp{};
-  itp.gp = batch_geom_params(t, d); itp.theta = d_theta; itp.n_theta = nth; itp.buf = buf;
+  itp.gp = batch_geom_params(t, d); itp.n_theta = nth;
   itp.part_a = part_a; itp.part_dl = part_dl; itp.part_f = part_f; itp.part_rp = part_rp;
   itp.n_feat = n_feat;
   const size_t smem_i = ItemSmem(d->max_layers, n_feat, t->n_species + 3 + d->n_tnodes).bytes();
@@ -1153,12 +1139,13 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   // One backward pass over `slots` wavenumber tiles per item: the tile kernel's partial sums,
   // their GPU-wide sum into each row's first slot, and the per-atmosphere kernel writing item b's
   // row r at grad + b * stride + r * nth.  No rows: one gradient with dL/dD from gd.
-  auto backward = [&](const RowGroup& rows, int slots, double* grad, long long stride) -> int {
+  auto backward = [&](int bc, const RowGroup& rows, int slots, double* grad,
+                      long long stride) -> int {
     const int n_rows = std::max(rows.n_rows, 1);
     ap.rows = rows; ap.tiles = slots;
     {
       KernelTimer kt(ctx, "k_adjoint_tile", s);
-      kern<<<dim3(slots, B), kAThreads, smem, s>>>(ap);
+      kern<<<dim3(slots, bc), kAThreads, smem, s>>>(ap);
       err = cudaGetLastError();
     }
     if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint tile kernel: ") + cudaGetErrorString(err));
@@ -1172,28 +1159,53 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
       ts.arr[2] = part_f;  ts.m[2] = (long long)d->max_layers * n_feat;
       ts.arr[3] = part_rp; ts.m[3] = 1;
       ts.slots = slots; ts.rows = rows;
-      const long long most = (long long)B * npad * npad;
+      const long long most = (long long)bc * npad * npad;
       const int gx = (int)std::max<long long>(1, std::min<long long>((most + 255) / 256, 8LL * n_sm));
-      k_adjoint_sum<<<dim3(gx, 4, n_rows), 256, 0, s>>>(ts, B);
+      k_adjoint_sum<<<dim3(gx, 4, n_rows), 256, 0, s>>>(ts, bc);
       err = cudaGetLastError();
       if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint sum kernel: ") + cudaGetErrorString(err));
     }
     itp.rows = rows; itp.slots = slots; itp.grad = grad; itp.item_stride = stride;
     {
       KernelTimer kt(ctx, "k_adjoint_item", s);
-      k_adjoint_item<<<dim3(B, n_rows), kItemThreads, smem_i, s>>>(itp);
+      k_adjoint_item<<<dim3(bc, n_rows), kItemThreads, smem_i, s>>>(itp);
       err = cudaGetLastError();
     }
     if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint item kernel: ") + cudaGetErrorString(err));
     return TR_OK;
   };
-  if (d_grad) {
-    RowGroup one;
-    one.n_rows = 0; one.first_bin = 0;
-    rc = backward(one, tiles, d_grad, nth);
-    if (rc != TR_OK) return rc;
-  }
-  if (d_jac) {
+  for (int b0 = 0; b0 < B; b0 += run) {
+    const int bc = std::min(run, B - b0);
+    const ItemBuffers rb = items_from(buf, b0, d->max_layers);
+    double* out = depth + (size_t)b0 * n_in;
+    double* bin_out = binned + (size_t)b0 * bins->dev.n_bin;
+    if (need_binned || use_kstore) {
+      rc = run_forward(ctx, t, d->max_layers, rb, bc, bins->dev.i0, n_in, out, n_in, precision, s,
+                       kbuf, dl16, &fc, /*opacity_only=*/!need_binned);
+      if (rc != TR_OK) return rc;
+    }
+    if (need_binned) {
+      KernelTimer kt(ctx, "k_bin", s);
+      err = launch_bin(bins->dev, bc, out, n_in, bins->dev.i0, bin_out, s);
+    }
+    if (err == cudaSuccess && d_grad) {
+      KernelTimer kt(ctx, "k_gd", s);
+      k_gd<<<dim3(bc, (n_in + kGdRun - 1) / kGdRun), kGdThreads, 0, s>>>(
+          bins->dev, bc, bin_out, d_obs, d_sigma_obs,
+          d_gbin ? d_gbin + (size_t)b0 * bins->dev.n_bin : nullptr, rb.items,
+          (d_gbin || !d_chi2) ? nullptr : d_chi2 + b0, gd, n_in);
+      err = cudaGetLastError();
+    }
+    if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
+    ap.f.buf = rb; itp.buf = rb; itp.theta = d_theta + (size_t)b0 * nth;
+    if (d_grad) {
+      RowGroup one;
+      one.n_rows = 0; one.first_bin = 0;
+      rc = backward(bc, one, tiles, d_grad + (size_t)b0 * nth, nth);
+      if (rc != TR_OK) return rc;
+    }
+    if (!d_jac) continue;
+    double* jac = d_jac + (size_t)b0 * bins->dev.n_bin * nth;
     // row k of dD_bin/dtheta: dL/dD is bin k's normalised weights, which vanish outside the
     // bin's native range, so a row covers only the tiles of that range.  The rows go in groups
     // of as many as the partial sums' space for one gradient (`tiles` slots per item) holds, one
@@ -1219,16 +1231,16 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
       if (g.n_rows == 0) {
         // a bin of more tiles than a group can list: its tiles one gradient-like pass, dL/dD
         // written to gd
-        k_row_gd<<<dim3((n_in + 255) / 256, B), 256, 0, s>>>(bins->dev, k, gd, n_in);
+        k_row_gd<<<dim3((n_in + 255) / 256, bc), 256, 0, s>>>(bins->dev, k, gd, n_in);
         err = cudaGetLastError();
         if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
-        rc = backward(g, tiles, d_jac + (size_t)k * nth, (long long)n_bin * nth);
+        rc = backward(bc, g, tiles, jac + (size_t)k * nth, (long long)n_bin * nth);
         if (rc != TR_OK) return rc;
         k0 = k + 1;
         continue;
       }
       g.slot0[g.n_rows] = (uint16_t)slots;
-      rc = backward(g, slots, d_jac + (size_t)k0 * nth, (long long)n_bin * nth);
+      rc = backward(bc, g, slots, jac + (size_t)k0 * nth, (long long)n_bin * nth);
       if (rc != TR_OK) return rc;
       k0 = k;
     }

@@ -179,6 +179,22 @@ constexpr int kOpxStride = 16;   // floats of per-item opacity weights (TR_MAX_M
 constexpr int kMaxZones = 2 * TR_MAX_MOL + 1;
 static_assert(TR_MAX_MOL + TR_MAX_CIA <= kOpxStride, "per-item opacity weights fit their stride");
 
+// Offset of row l in the packed path-length layout (row l holds rays 0 .. pad8(l+1)-1):
+// sum_{k<l} pad8(k+1) = 8 (q+1)(4q + r) with l = 8q + r.
+__host__ __device__ inline int dlp_offset(int l) {
+  const int q = l >> 3, r = l & 7;
+  return 8 * (q + 1) * (4 * q + r);
+}
+
+// The same buffers from item b0 on.
+inline ItemBuffers items_from(ItemBuffers b, int b0, int max_layers) {
+  const size_t n = (size_t)b0, m = n * max_layers;
+  b.layers += m; b.z += m + n; b.tl += m; b.zf += m + n; b.op += 2 * m;
+  b.opx += n * kMaxZones * kOpxStride; b.dlt += m * b.npad; b.dlp += n * dlp_offset(max_layers);
+  b.aj += n * b.npad; b.rayc += n * kMaxZones * TR_MAX_SPECIES; b.items += n;
+  return b;
+}
+
 // Launchers (stream-ordered; return cudaGetLastError()).
 // k_profile (per-atmosphere set-up: everything the opacity kernels read), k_altitude (the
 // hydrostatic altitudes and annulus weights, from the inputs k_profile leaves in the altitude
@@ -204,13 +220,6 @@ constexpr int kOpacityTile = 256;
 constexpr int kRowTile = 256;
 // Wavenumbers per work unit of the fused forward kernel (the inner box of its tensor maps).
 constexpr int kFusedTile = 128;
-
-// Offset of row l in the packed path-length layout (row l holds rays 0 .. pad8(l+1)-1):
-// sum_{k<l} pad8(k+1) = 8 (q+1)(4q + r) with l = 8q + r.
-__host__ __device__ inline int dlp_offset(int l) {
-  const int q = l >> 3, r = l & 7;
-  return 8 * (q + 1) * (4 * q + r);
-}
 
 struct FwdParams {
   const float* sigma; int n_mol, n_p, n_t, wn_pad;

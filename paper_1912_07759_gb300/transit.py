@@ -470,8 +470,7 @@ def adjoint_transit(ctx: TransitContext, tables: XsecTables, spec: BatchSpec,
     binned spectrum) as a fifth value.  With gbin the gradient is the vector-Jacobian product
     gbin . dD_bin/dtheta, else the chi^2 gradient (obs, sigma_obs needed); want_grad=False
     (with want_jac=True) computes only the Jacobian.  recompute_k: 1 recomputes the opacity in
-    the backward pass; -1 (or 0) reuses the forward's when the workspace's K buffer holds the
-    whole batch."""
+    the backward pass; -1 (or 0) reuses the forward's."""
     B = int(theta.shape[0])
     dev = theta.device
     if not want_grad and not want_jac:
