@@ -8,25 +8,36 @@
 //
 // k_contract_tc: persistent, one CTA per SM over a contiguous range of (item, 128-wn) units.
 // A unit's layers are taken as two halves (the top half first): each half is a job of its own
-// for the splitters and the MMA, so the split of one half overlaps the MMAs of the one before.
+// for the loads, the splitters and the MMA, so the loads of later halves, the split of one half
+// and the MMAs of the one before overlap.
 // The kernel is instantiated per padded layer count, so the MMA issue and split loops are
 // unrolled with constant operands: issued from a runtime loop, the MMAs went at about half the
 // rate (the issuing thread, not the tensor pipe, set the pace).
 // Warp roles, every hand-over through an mbarrier:
-//   * warp 8 (producer): TMA loads of the unit's FP32 K tile [KP layers][128 wn] (boxes of 8
-//     rows of the opacity kernel's K buffer) into one of two stages;
-//   * warps 0-3 and 10-13 (splitters; thread = TMEM lane = one wavenumber of the unit, the two
-//     warps of a lane quarter taking alternate 8-layer groups): when the item changes (once
-//     every MMA of the previous unit is done), one thread bulk-copies the item's path-length
-//     tiles DL_hi / DL_lo (rays x layers, K-major core matrices, built once per item by
-//     k_dl_tf32) into shared memory; per half, each thread splits its wavenumber's K values of
-//     the half's layers (zero at and beyond N) and stores K_hi and K_lo into one of two TMEM
-//     half buffers (the MMA's A operand, column = layer);
+//   * warp 8 (producer): TMA loads of a half's FP32 K rows [KP / 2 layers][128 wn] (boxes of 8
+//     rows of the opacity kernel's K buffer) into a ring of up to eight half-unit stages;
+//   * warps 0-3 and 10-13 (splitters; thread = TMEM lane = one wavenumber of the unit; the first
+//     four take the top halves, the others the bottom halves, side by side): per half, each
+//     thread splits its wavenumber's K values of the half's layers (zero at and beyond N) and
+//     stores K_hi and K_lo into its half's TMEM buffer (the MMA's A operand, column = layer);
+//     when the item changes (once every MMA of the previous unit is done), one thread
+//     bulk-copies the item's path-length tiles DL_hi / DL_lo (built once per item by k_dl_tf32)
+//     into shared memory;
 //   * warp 9 (one thread): per half, for its 8-layer slices from the top down, three MMAs
 //     D[128 x N_ks] (+)= A[128 x 8] B[N_ks x 8]^T, N_ks the rays the slice reaches (DL = 0 for
 //     rays above a layer), into the unit's one of two TMEM accumulators; a commit frees the
 //     half buffer, one after the bottom half hands the accumulator to the epilogue;
 //   * warps 4-7 (epilogue): tau from TMEM -> sum_j a_j (1 - e^-tau_j) -> FP64 depth.
+// What sets the pace, 100 layers x 200,000 wavenumbers (10.3 units of 112 x 128 an SM; K read at
+// the copy bandwidth would take 11.8 us): 30.6 us an atmosphere in batches of 64 at first, 27.7
+// with the path-length tiles cut to the rays each slice reaches (57 KB instead of 100), which
+// makes room for six half-unit stages (two whole-unit stages were refilled a unit late), 21.0 with
+// the MMA thread elected by elect.sync and its descriptors moved by constants (the issuing
+// thread's operand moves took about 100 cycles an MMA, the tensor pipe 32), 19.0 with the halves
+// split side by side (the split alone took 3,000 cycles a unit, mostly waits), 18.8 with the
+// epilogue's TMEM loads one step ahead.  One atmosphere: 42.6 -> 28.6 us.  Left: without the
+// epilogue 14.3 (its exponentials share the SM with the split), without the MMAs 16.2.  Two CTAs
+// per SM with 32-layer chunks took 23.3; a second epilogue group 22.2 (spills).
 // All waits are bounded; on a timeout every role stops, in-flight copies and MMAs are waited
 // for (bounded) and the TMEM is released before the CTA exits.
 #include <algorithm>
@@ -42,7 +53,7 @@ constexpr int kTEpi0 = 4;                 // epilogue warps 4..7
 constexpr int kTProd = 8;
 constexpr int kTMma = 9;
 constexpr int kTSplit1 = 10;              // splitters: warps 0..3 and 10..13
-constexpr int kTSplitters = 8;
+constexpr int kTSplitters = 4;            // warps per half: 0..3 the top halves, 10..13 the bottom
 constexpr int kTThreads = 32 * (kTSplit1 + 4);
 constexpr int kTMaxKP = 112;              // layers (padded to 16) the kernel takes
 // TMEM columns: half buffer h at 128 h (K_hi at + 0, K_lo at + 64, KP / 2 columns each);
@@ -51,13 +62,28 @@ constexpr uint32_t kColHalf = 128, kColLo = 64, kColD0 = 256, kColD1 = 384, kTme
 
 __host__ __device__ inline int pad16i(int n) { return (n + 15) & ~15; }
 
+// Rays slice ks (layers 8 ks .. 8 ks + 7) reaches: j <= 8 ks + 7, rounded up to the MMA's N step
+// of 16; slices 2 m and 2 m + 1 both 16 (m + 1).  A slice's path-length tile is its rays x 8
+// layers in K-major core matrices (8 rays x 4 layers, 128 bytes): ray group g, layer half c at
+// 128 (2 g + c).  Core matrices before slice ks: dl_cores(ks).
+__host__ __device__ constexpr int dl_cores(int ks) {
+  return 4 * (ks / 2) * (ks / 2 + 1) + (ks & 1) * 4 * (ks / 2 + 1);
+}
+
+constexpr int kTMaxStages = 8;
 struct TcLayout {
-  uint32_t stage, dl, aj, total;
-  __host__ __device__ TcLayout(int KP, int NP) {
-    stage = (uint32_t)KP * kTM * 4;                       // FP32 K tile [KP][128]
-    dl = 2 * stage;                                       // DL_hi, DL_lo [NP][KP] TF32
-    aj = dl + 2u * (uint32_t)NP * KP * 4;
-    total = aj + 2u * kTM * 4 + 128u;                     // + alignment slack
+  uint32_t stage, dl_bytes, dl, aj, total;
+  int stages;
+  __host__ __device__ TcLayout(int KP) {
+    stage = (uint32_t)(KP / 2) * kTM * 4;                 // FP32 K rows of a half [KP / 2][128]
+    dl_bytes = (uint32_t)dl_cores(KP / 8) * 128u;         // DL_hi; DL_lo follows
+    const uint32_t rest = 2 * dl_bytes + 2u * kTM * 4 + 128u;   // + alignment slack
+    constexpr uint32_t kDyn = 227u * 1024u - 256u;        // less the static shared memory
+    stages = (int)((kDyn - rest) / stage);
+    if (stages > kTMaxStages) stages = kTMaxStages;
+    dl = (uint32_t)stages * stage;
+    aj = dl + 2 * dl_bytes;
+    total = dl + rest;
   }
 };
 
@@ -68,26 +94,29 @@ __device__ __forceinline__ float tf32_hi(float x) {
 }
 
 // The path-length tiles of every item, the MMA's B operand: tiles[b][0] = DL_hi, [b][1] =
-// DL_lo, each [NP rays][KP layers] in the K-major core-matrix layout (core matrix m = (j / 8) *
-// (KP / 4) + l / 4 of 8 rays x 4 layers, 128 bytes, row j % 8, column l % 4), zero for j > l and
+// DL_lo, each the slices' core matrices (see dl_cores; row j % 8, column l % 4), zero for j > l and
 // outside the item's N layers.  Grid (core matrices / 4, B items): a warp writes one core
 // matrix per store (lane = (ray, layer) of it, one value each) from four 32-byte row segments
 // of the geometry kernel's layer-major DL.
 __global__ void __launch_bounds__(128)
-k_dl_tf32(ItemBuffers buf, int max_layers, int NP, int KP, float* __restrict__ tiles) {
+k_dl_tf32(ItemBuffers buf, int max_layers, int n_cm, float* __restrict__ tiles) {
   const int b = blockIdx.y;
-  const int cm_k = KP / 4, n_cm = (NP / 8) * cm_k;
-  const int m = 4 * blockIdx.x + (threadIdx.x >> 5);        // core matrix of this warp
-  if (m >= n_cm) return;
+  const int q = 4 * blockIdx.x + (threadIdx.x >> 5);        // core matrix of this warp
+  if (q >= n_cm) return;
+  int m = 0;                                                // its pair of slices
+  while (4 * (m + 1) * (m + 2) <= q) ++m;
+  int rem = q - 4 * m * (m + 1);
+  const int odd = rem >= 4 * (m + 1) ? 1 : 0;
+  rem -= odd * 4 * (m + 1);
   const int lane = threadIdx.x & 31, r = lane >> 2, c = lane & 3;
-  const int j = 8 * (m / cm_k) + r, l = 4 * (m % cm_k) + c;
+  const int j = 8 * (rem >> 1) + r, l = 8 * (2 * m + odd) + 4 * (rem & 1) + c;
   const int N = buf.items[b].n_layers;
   const float* dlt = buf.dlt + (size_t)b * max_layers * buf.npad;
   const float x = (l < N && j <= l) ? __ldg(dlt + (size_t)l * buf.npad + j) : 0.f;
   const float h = tf32_hi(x);
-  float* hi = tiles + (size_t)b * 2 * NP * KP;
-  hi[(size_t)m * 32 + lane] = h;                            // row r, column c: 4 r + c = lane
-  hi[(size_t)NP * KP + (size_t)m * 32 + lane] = x - h;
+  float* hi = tiles + ((size_t)b * 2 * n_cm + q) * 32;
+  hi[lane] = h;                                             // row r, column c: 4 r + c = lane
+  hi[(size_t)n_cm * 32 + lane] = x - h;
 }
 
 // Barrier over `threads` threads (named barrier `id`) that also returns whether any of them
@@ -111,16 +140,17 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
               const float* __restrict__ tiles) {
   constexpr int NP = KP;                    // rays (padded) = layers (padded)
   extern __shared__ __align__(128) uint8_t tsm_raw[];
-  __shared__ __align__(8) uint64_t sfull[2], sempty[2], hfull[2], hfree[2], accfull[2],
-      accempty[2], dlfull;
+  __shared__ __align__(8) uint64_t sfull[kTMaxStages], sempty[kTMaxStages], hfull[2], hfree[2],
+      accfull[2], accempty[2], dlfull;
   __shared__ uint32_t tmem_base;
   __shared__ int abort_flag;
   const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
   uint8_t* base = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(tsm_raw) + 127) &
                                              ~(uintptr_t)127);
-  const TcLayout lay(KP, NP);
+  const TcLayout lay(KP);
+  const int S = lay.stages;
   uint8_t* B_hi = base + lay.dl;
-  uint8_t* B_lo = B_hi + (size_t)NP * KP * 4;
+  uint8_t* B_lo = B_hi + lay.dl_bytes;
   float* ep_aj = reinterpret_cast<float*>(base + lay.aj);      // [2][128], epilogue's copy
   const long long units = (long long)Bc * n_tiles;
   const long long per = (units + gridDim.x - 1) / gridDim.x;
@@ -132,8 +162,8 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
 
   if (warp == 0) tmem_alloc(&tmem_base, kTmemCols);
   if (tid == 0) {
+    for (int i = 0; i < S; ++i) { mbar_init(&sfull[i], 1); mbar_init(&sempty[i], kTSplitters); }
     for (int i = 0; i < 2; ++i) {
-      mbar_init(&sfull[i], 1); mbar_init(&sempty[i], kTSplitters);
       mbar_init(&hfull[i], kTSplitters); mbar_init(&hfree[i], 1);
       mbar_init(&accfull[i], 1); mbar_init(&accempty[i], 4);
     }
@@ -151,104 +181,93 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
   if (warp == kTProd) {
     // ---------------- producer
     if (lane == 0) {
-      int k = 0;
-      for (; k < n_units; ++k) {
-        const long long u = u_begin + k;
-        const int bc = (int)(u / n_tiles), tile = (int)(u % n_tiles);
-        const int s = k & 1, q = k >> 1;
+      // half job h = 2k + (1 - hh): the rows of half hh (top half first) of unit k
+      const int n_jobs = 2 * n_units;
+      int h = 0, st = 0, q = 0;
+      for (; h < n_jobs; ++h) {
+        const long long u = u_begin + (h >> 1);
+        const int row0 = (int)u * p.max_layers + ((h & 1) ? 0 : HL);   // u = bc n_tiles + tile
         const bool ok = q == 0 ||
-                        mbar_wait_bounded(&sempty[s], (q - 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
+                        mbar_wait_bounded(&sempty[st], (q - 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
         if (!ok || *(volatile int*)&abort_flag) { atomicExch(&abort_flag, 1); break; }
-        uint8_t* st = base + s * lay.stage;
-        mbar_arrive_expect_tx(&sfull[s], lay.stage);
-        for (int i = 0; i < KP / 8; ++i)
-          tma_load_2d(st + (size_t)i * 8 * kTM * 4, &tm_k, 0,
-                      (bc * n_tiles + tile) * p.max_layers + i * 8, &sfull[s]);
+        uint8_t* sb = base + (size_t)st * lay.stage;
+        mbar_arrive_expect_tx(&sfull[st], lay.stage);
+        for (int i = 0; i < HL / 8; ++i)
+          tma_load_2d(sb + (size_t)i * 8 * kTM * 4, &tm_k, 0, row0 + i * 8, &sfull[st]);
+        if (++st == S) { st = 0; ++q; }
       }
-      for (int i = 0; i < 2 && i < k; ++i) {      // every copy issued has landed
-        const int kl = k - 1 - i;
-        mbar_wait_bounded(&sfull[kl & 1], (kl >> 1) & 1, nullptr, 0);
+      for (int i = 0; i < S && i < h; ++i) {      // every copy issued has landed
+        const int hl = h - 1 - i;
+        mbar_wait_bounded(&sfull[hl % S], (hl / S) & 1, nullptr, 0);
       }
     }
   } else if (warp < kTEpi0 || warp >= kTSplit1) {
     // ---------------- splitters: thread v = wavenumber row v of the unit = TMEM lane v
     const int v = 32 * (warp & 3) + lane;          // 0 .. 127
     const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
-    const int g0 = warp >= kTSplit1 ? 1 : 0;      // the two warps of a lane quarter take
-                                                   // alternate 8-layer groups
-    const uint32_t tile_bytes = (uint32_t)NP * KP * 4;
+    const int hb = warp >= kTSplit1 ? 1 : 0;       // half job parity: 0 top halves, 1 bottom
+    const int l0 = hb ? 0 : HL;                    // the half's first layer
+    const bool lead = tid == 32 * kTSplit1;        // copies the items' path-length tiles
     int dl_item = -1, dl_issued = 0;
+    int st = hb, sq = 0;                           // stage of half job 2k + hb
+    while (st >= S) { st -= S; ++sq; }
     for (int k = 0; k < n_units; ++k) {
       const long long u = u_begin + k;
       const int b = p.b_off + (int)(u / n_tiles);
       const int N = __ldg(&p.buf.items[b].n_layers);
-      const int s = k & 1;
-      if (b != dl_item) {
-        // the item's path-length tiles replace the old ones once every MMA of unit k-1 is done
-        // (the commit of its bottom half, half job 2k - 1, completes after all of them; the
-        // splitters have waited for the commit of half job 2k - 3 before splitting unit k-1,
-        // so this barrier is at most one phase behind the one waited for)
-        bool dok = k == 0 || mbar_wait_bounded(&hfree[1], (k - 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
-        dok = dok && !*(volatile int*)&abort_flag;
-        if (tc_sync_or(1, 32 * kTSplitters, !dok)) { if (lane == 0) atomicExch(&abort_flag, 1); break; }
-        // one thread starts the copy; the MMA thread waits for it (the split does not need it)
-        if (tid == 0) {
-          const float* src = tiles + (size_t)b * 2 * NP * KP;
-          mbar_arrive_expect_tx(&dlfull, 2u * tile_bytes);
-          bulk_g2s(B_hi, src, tile_bytes, &dlfull);
-          bulk_g2s(B_lo, src + (size_t)NP * KP, tile_bytes, &dlfull);
-        }
+      // half job 2k + hb: the MMAs of half job 2k - 2 + hb are done with its half buffer
+      bool hok = (k == 0 || mbar_wait_bounded(&hfree[hb], (k - 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT)) &&
+                 !*(volatile int*)&abort_flag;
+      // when the item changes, its path-length tiles replace the old ones once every MMA of unit
+      // k - 1 is done: the commit of its bottom half, just waited for by the bottom halves'
+      // splitters, completes after all of them.  The MMA thread waits for the copy
+      if (lead && hok && b != dl_item) {
+        const char* src = reinterpret_cast<const char*>(tiles) + (size_t)b * 2 * lay.dl_bytes;
+        mbar_arrive_expect_tx(&dlfull, 2u * lay.dl_bytes);
+        bulk_g2s(B_hi, src, lay.dl_bytes, &dlfull);
+        bulk_g2s(B_lo, src + lay.dl_bytes, lay.dl_bytes, &dlfull);
         ++dl_issued;
         dl_item = b;
       }
-      // the unit's K tile has landed
-      const bool ok = mbar_wait_bounded(&sfull[s], (k >> 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT) &&
-                      !*(volatile int*)&abort_flag;
-      if (tc_sync_or(1, 32 * kTSplitters, !ok)) { if (lane == 0) atomicExch(&abort_flag, 1); break; }
-      const float* kf = reinterpret_cast<const float*>(base + s * lay.stage);
-      bool stop = false;
-      for (int hh = 1; hh >= 0; --hh) {
-        // half job h = 2k + (1 - hh) (the top half first) into half buffer h & 1, once the MMAs
-        // of half job h - 2 are done with it
-        const int h = 2 * k + (1 - hh), hb = h & 1, hq = h >> 1;
-        bool hok = hq == 0 || mbar_wait_bounded(&hfree[hb], (hq - 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
-        hok = hok && !*(volatile int*)&abort_flag;
-        if (tc_sync_or(1, 32 * kTSplitters, !hok)) { if (lane == 0) atomicExch(&abort_flag, 1); stop = true; break; }
-        tcgen05_fence_after();
-        const uint32_t col = tmem + lane_base + kColHalf * hb;
-#pragma unroll
-        for (int gg = 0; gg < (HL / 8 + 1) / 2; ++gg) {
-          const int g = 2 * gg + g0;
-          if (g >= HL / 8) break;
-          uint32_t hi[8], lo[8];
-#pragma unroll
-          for (int i = 0; i < 8; ++i) {
-            const int l = hh * HL + 8 * g + i;
-            const float x = l < N ? kf[l * kTM + v] : 0.f;
-            const float hv = tf32_hi(x);
-            hi[i] = __float_as_uint(hv);
-            lo[i] = __float_as_uint(x - hv);
-          }
-          tmem_st8(col + 8 * g, hi);
-          tmem_st8(col + kColLo + 8 * g, lo);
-        }
-        tmem_st_wait();
-        tcgen05_fence_before();
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&hfull[hb]);     // this warp's rows of the half are written
-      }
-      if (stop) break;
       __syncwarp();
-      if (lane == 0) mbar_arrive(&sempty[s]);       // this warp's reads of the stage are done
+      // its K rows have landed
+      hok = hok && mbar_wait_bounded(&sfull[st], sq & 1, p.dev_err, TR_DEVERR_TIMEOUT);
+      if (!__all_sync(0xffffffffu, hok)) { if (lane == 0) atomicExch(&abort_flag, 1); break; }
+      tcgen05_fence_after();
+      const float* kf = reinterpret_cast<const float*>(base + (size_t)st * lay.stage);
+      const uint32_t col = tmem + lane_base + kColHalf * hb;
+      const int n_half = N - l0;                     // layers of the half below the item's top
+#pragma unroll
+      for (int g = 0; g < HL / 8; ++g) {
+        uint32_t hi[8], lo[8];
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const int l = 8 * g + i;
+          const float x = l < n_half ? kf[l * kTM + v] : 0.f;
+          const float hv = tf32_hi(x);
+          hi[i] = __float_as_uint(hv);
+          lo[i] = __float_as_uint(x - hv);
+        }
+        tmem_st8(col + 8 * g, hi);
+        tmem_st8(col + kColLo + 8 * g, lo);
+      }
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&sempty[st]);      // this warp's reads of the stage are done
+      st += 2;
+      while (st >= S) { st -= S; ++sq; }
+      tmem_st_wait();
+      tcgen05_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(&hfull[hb]);       // this warp's rows of the half are written
     }
     // the last tile copy has landed before the CTA may exit (the MMA thread observes every copy
     // but the last one when the CTA stops early)
-    if (tid == 0 && dl_issued > 0) mbar_wait_bounded(&dlfull, (dl_issued - 1) & 1, nullptr, 0);
+    if (dl_issued > 0) mbar_wait_bounded(&dlfull, (dl_issued - 1) & 1, nullptr, 0);
   } else if (warp == kTMma) {
     // ---------------- MMA issue (one thread)
-    if (lane == 0) {
-      const uint32_t sbo = (uint32_t)(KP / 4) * 128;
-      const uint32_t bh = smem_addr(B_hi), bl = smem_addr(B_lo);
+    if (elect_one()) {
+      const uint64_t dh0 = umma_smem_desc(smem_addr(B_hi), 128, 256);
+      const uint64_t dl0 = umma_smem_desc(smem_addr(B_lo), 128, 256);
       uint64_t* last = nullptr;                     // the last commit issued and its phase
       int last_par = 0, dl_item = -1, dl_copies = 0;
       bool stop = false;
@@ -281,9 +300,8 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
             // the rays slice ks reaches: j <= 8 ks + 7, rounded up to the MMA's N step of 16
             const int n = min(NP, pad16i(8 * ks + 8));
             const uint32_t idesc = umma_idesc_tf32_f32(kTM, n);
-            const uint32_t koff = (uint32_t)ks * 256;          // two core matrices along K
-            const uint64_t dh = umma_smem_desc(bh + koff, 128, sbo);
-            const uint64_t dlo = umma_smem_desc(bl + koff, 128, sbo);
+            const uint64_t koff = (uint64_t)dl_cores(ks) * (128 / 16);
+            const uint64_t dh = dh0 + koff, dlo = dl0 + koff;
             umma_tf32_ta(d, ah + 8 * i, dh, idesc, first ? 0u : 1u);
             umma_tf32_ta(d, ah + 8 * i, dlo, idesc, 1u);
             umma_tf32_ta(d, al + 8 * i, dh, idesc, 1u);
@@ -299,11 +317,10 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
       // issued completes after all of them)
       if (last) mbar_wait_bounded(last, (uint32_t)last_par, nullptr, 0);
     }
-  } else if (warp < kTProd) {
+  } else {
     // ---------------- epilogue: thread = TMEM lane = wavenumber row
-    const int q4 = warp - kTEpi0;
-    const int row = 32 * q4 + lane;
-    const uint32_t lane_base = (uint32_t)(32 * q4) << 16;
+    const int row = 32 * (warp & 3) + lane;
+    const uint32_t lane_base = (uint32_t)(32 * (warp & 3)) << 16;
     for (int k = 0; k < n_units; ++k) {
       const long long u = u_begin + k;
       const int bc = (int)(u / n_tiles), tile = (int)(u % n_tiles);
@@ -318,13 +335,23 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
       if (tc_sync_or(2, 128, !ok)) { if (lane == 0) atomicExch(&abort_flag, 1); break; }
       tcgen05_fence_after();
       const uint32_t taddr = tmem + lane_base + (a ? kColD1 : kColD0);
+      // 16 columns are read while the 16 before are summed
       float part = 0.f;
+      uint32_t t[2][16];
+      tmem_ld16_nowait(taddr, t[0]);
 #pragma unroll
       for (int c0 = 0; c0 < NP; c0 += 16) {
-        float tau[16];
-        tmem_ld16(taddr + (uint32_t)c0, tau);
+        uint32_t* tau = t[(c0 / 16) & 1];
+        tmem_ld_wait16(tau);
+        if (c0 + 16 < NP) tmem_ld16_nowait(taddr + (uint32_t)(c0 + 16), t[(c0 / 16 + 1) & 1]);
 #pragma unroll
-        for (int i = 0; i < 16; ++i) part = fmaf(aj[c0 + i], 1.f - __expf(-tau[i]), part);
+        for (int i = 0; i < 16; i += 4) {
+          const float4 w = *reinterpret_cast<const float4*>(aj + c0 + i);
+          part = fmaf(w.x, 1.f - __expf(-__uint_as_float(tau[i])), part);
+          part = fmaf(w.y, 1.f - __expf(-__uint_as_float(tau[i + 1])), part);
+          part = fmaf(w.z, 1.f - __expf(-__uint_as_float(tau[i + 2])), part);
+          part = fmaf(w.w, 1.f - __expf(-__uint_as_float(tau[i + 3])), part);
+        }
       }
       tcgen05_fence_before();
       __syncwarp();
@@ -344,31 +371,29 @@ k_contract_tc(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int
 
 size_t tc_dl_bytes(int B, int max_layers) {
   if (!tc_contract_fits(max_layers)) return 0;
-  const size_t P = (size_t)pad16i(max_layers);
-  return sizeof(float) * 2 * (size_t)B * P * P;
+  return 2 * (size_t)B * TcLayout(pad16i(max_layers)).dl_bytes;
 }
 
 cudaError_t launch_dl_tf32(const ItemBuffers& buf, int B, int max_layers, void* tiles,
                            cudaStream_t s) {
   if (B <= 0) return cudaSuccess;
   if (!tc_contract_fits(max_layers)) return cudaErrorInvalidValue;
-  const int P = pad16i(max_layers);
-  const int n_cm = (P / 8) * (P / 4);
-  k_dl_tf32<<<dim3((n_cm + 3) / 4, B), 128, 0, s>>>(buf, max_layers, P, P,
+  const int n_cm = dl_cores(pad16i(max_layers) / 8);
+  k_dl_tf32<<<dim3((n_cm + 3) / 4, B), 128, 0, s>>>(buf, max_layers, n_cm,
                                                     static_cast<float*>(tiles));
   return cudaGetLastError();
 }
 
 bool tc_contract_fits(int max_layers) {
   const int KP = pad16i(max_layers);
-  return max_layers >= 1 && KP <= kTMaxKP && TcLayout(KP, KP).total <= 227u * 1024u;
+  return max_layers >= 1 && KP <= kTMaxKP;
 }
 
 cudaError_t launch_contract_tc(const FwdParams& p, int Bc, const float* kbuf, const void* tiles,
                                cudaStream_t s) {
   if (Bc <= 0 || p.wn_count <= 0) return cudaSuccess;
   if (!tc_contract_fits(p.max_layers)) return cudaErrorInvalidValue;
-  const int KP = pad16i(p.max_layers), NP = KP;
+  const int KP = pad16i(p.max_layers);
   const int w_first = wn_first(p.wn_begin);
   if (!tiles) return cudaErrorInvalidValue;
   const int tiles_w = (p.wn_begin + p.wn_count - w_first + kTM - 1) / kTM;
@@ -376,7 +401,7 @@ cudaError_t launch_contract_tc(const FwdParams& p, int Bc, const float* kbuf, co
   if (!encode_2d_f32(&tm, kbuf, kTM, (unsigned long long)Bc * tiles_w * p.max_layers, kTM * 4, kTM,
                      8))
     return cudaErrorInvalidValue;
-  const uint32_t smem = TcLayout(KP, NP).total;
+  const uint32_t smem = TcLayout(KP).total;
   void (*kern)(FwdParams, CUtensorMap, int, int, const float*) = nullptr;
   switch (KP) {
     case 16: kern = k_contract_tc<16>; break;

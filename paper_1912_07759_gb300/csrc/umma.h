@@ -60,6 +60,18 @@ __host__ __device__ inline uint32_t umma_idesc_tf32_f32(int M, int N) {
 }
 
 #ifdef __CUDACC__
+// True in one lane of the (converged) warp.  The compiler knows that a single thread takes the
+// branch, so operands of the MMA instructions inside stay in uniform registers.
+__device__ __forceinline__ bool elect_one() {
+  uint32_t p;
+  asm volatile(
+      "{\n\t.reg .pred p;\n\t"
+      "elect.sync _|p, 0xffffffff;\n\t"
+      "selp.u32 %0, 1, 0, p;\n\t}"
+      : "=r"(p));
+  return p != 0;
+}
+
 __device__ __forceinline__ void tmem_alloc(uint32_t* dst_smem, uint32_t ncols) {
   asm volatile("tcgen05.alloc.cta_group::1.sync.aligned.shared::cta.b32 [%0], %1;"
                :: "r"(static_cast<uint32_t>(__cvta_generic_to_shared(dst_smem))), "r"(ncols)
@@ -139,7 +151,7 @@ __device__ __forceinline__ void umma_bf16_ta(uint32_t d_tmem, uint32_t a_tmem, u
       :: "r"(d_tmem), "r"(a_tmem), "l"(b_desc), "r"(idesc), "r"(accumulate) : "memory");
 }
 
-// 16 consecutive FP32 columns of this thread's TMEM lane without waiting (tmem_ld_wait
+// 16 consecutive FP32 columns of this thread's TMEM lane without waiting (tmem_ld_wait16
 // completes the warp's loads; the registers must not be read before it).
 __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
   asm volatile(
@@ -150,8 +162,14 @@ __device__ __forceinline__ void tmem_ld16_nowait(uint32_t taddr, uint32_t* r) {
         "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
       : "r"(taddr) : "memory");
 }
-__device__ __forceinline__ void tmem_ld_wait() {
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+// Completes the warp's TMEM loads; r, a register set of tmem_ld16_nowait, passes through so that
+// no use of it can be scheduled before the wait.
+__device__ __forceinline__ void tmem_ld_wait16(uint32_t* r) {
+  asm volatile("tcgen05.wait::ld.sync.aligned;"
+               : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]),
+                 "+r"(r[7]), "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]),
+                 "+r"(r[13]), "+r"(r[14]), "+r"(r[15])
+               :: "memory");
 }
 
 // Store 8 consecutive 32-bit columns of this thread's TMEM lane (no wait).
