@@ -25,6 +25,7 @@
 #include <cmath>
 #include <cstddef>
 #include <cuda_fp16.h>
+#include <type_traits>
 #include "tma.h"
 #include "tr_internal.h"
 
@@ -61,6 +62,7 @@ struct AdjParams {
   const double* inv_dtc;          // [n_t_cia - 1]
   const float* gd;                // [B][n_in] dL/dD at the native wavenumbers of the range
   int n_in, tiles, n_feat;        // tiles: slots per item of the partial sums
+  unsigned ray_mask;              // species with Rayleigh cross-sections that are not all zero
   float* part_a;                  // [B][tiles][npad]
   float* part_dl;                 // [B][tiles][npad][npad]  (ray j, shell l), j <= l
   float* part_f;                  // [B][tiles][max_layers][n_feat]
@@ -143,6 +145,29 @@ __device__ __forceinline__ float2 sig2(const FwdParams& p, int m, size_t off) {
   }
 }
 
+// The same pair as loaded, so that it can be fetched ahead of its use, and its packed value.
+template <bool F16>
+using SigRaw = std::conditional_t<F16, unsigned, unsigned long long>;
+template <bool F16>
+__device__ __forceinline__ SigRaw<F16> sig_fetch(const FwdParams& p, size_t off) {
+  if constexpr (F16)
+    return __ldg(reinterpret_cast<const unsigned*>(reinterpret_cast<const __half*>(p.logsig16) + off));
+  else
+    return __ldg(reinterpret_cast<const unsigned long long*>(p.sigma + off));
+}
+template <bool F16>
+__device__ __forceinline__ unsigned long long sig_value(SigRaw<F16> v, float c) {
+  if constexpr (F16) {
+    const float2 f = __half22float2(*reinterpret_cast<const __half2*>(&v));
+    float a, b;
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(a) : "f"((f.x + c) * kLog2Of10a));
+    asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(b) : "f"((f.y + c) * kLog2Of10a));
+    return pack2(a, b);
+  } else {
+    return v;
+  }
+}
+
 __device__ __forceinline__ float warp_sum(float v) {
 #pragma unroll
   for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
@@ -165,66 +190,81 @@ __device__ __forceinline__ float2 rayleigh_sum2(const FwdParams& p, int b, int w
   return ray;
 }
 
-// floats per feature row of a warp's reduction buffer: a multiple of 4 (rows read as float4)
-// with rows 4 banks apart, so neither the lanes' column writes nor the 8-lane phases of the
-// float4 row reads conflict
-constexpr int kRedPitch = 36;
+// A warp sums the features of its tile's kRT layers two at a time: kRedRows = 2 kRT rows of one
+// term per lane.  The pitch (floats) keeps rows 8-byte aligned and 2 banks apart: the lanes' writes
+// along a row and the reads of 16 bytes of each row (two wavefronts) do not conflict.
+constexpr int kRedPitch = 34, kRedRows = 2 * kRT;
+constexpr int kHdr = 12;    // floats of a layer's header: tt, tt, tp, tp, 1/dT, 1/dT, cell, CIA bracket, ttc, 1/dTc
 
+// Dynamic shared memory of a CTA that leaves room for three on an SM (228 KB less 1 KB and the
+// rounding of each): up to 101 layers
+constexpr size_t kThreeCtaSmem = (228u * 1024u) / 3 - 1024u - 128u;
+
+// Shared memory of a tile.  The path lengths are the packed rows of ItemBuffers::dlp (row l
+// holds rays 0 .. pad8(l+1)-1, zero for j > l); the G_K phase may read up to kRT - 1 rows past
+// layer N's, inside the arrays that follow, for layers that it does not use.
 struct AdjSmem {
-  int npad, kt_rows, n_feat;
-  // the tile's Rayleigh rows (layer-independent) are staged once: TR_MAX_SPECIES x kAT floats
-  __host__ __device__ AdjSmem(int max_layers, int nf)
-      : npad(pad8(max_layers)), kt_rows(max_layers), n_feat(nf) {}
-  // the warps' reduction buffers of the feature phase reuse the K tile's space (K is not
-  // read after the G_DL phase) when they fit there, else follow the other buffers
-  __host__ __device__ size_t red_floats() const { return (size_t)kAWarps * n_feat * kRedPitch; }
-  __host__ __device__ bool red_in_kt() const { return red_floats() <= (size_t)kt_rows * kAT; }
+  int npad, kt_rows, n_act, n_ray;
+  __host__ __device__ AdjSmem(int max_layers, int na, int nr)
+      : npad(pad8(max_layers)), kt_rows(max_layers), n_act(na), n_ray(nr) {}
+  // a warp's feature buffers: term rows, layer headers, sums.  They reuse the K tile's space (K
+  // is not read after the G_DL phase) when they fit there, else follow the other buffers
+  __host__ __device__ size_t red_floats() const { return kRedRows * kRedPitch + kHdr * kRT + (size_t)((kRT * n_act + 3) & ~3); }
+  __host__ __device__ bool red_in_kt() const { return kAWarps * red_floats() <= (size_t)kt_rows * kAT; }
+  __host__ __device__ size_t dl_floats() const { return dlp_offset(kt_rows); }
+  // the tile's Rayleigh rows (layer-independent) are staged once: n_ray x kAT floats
   __host__ __device__ size_t floats() const {
-    return (size_t)kt_rows * kAT + (size_t)npad * npad + npad + (size_t)npad * kAT + kAT +
-           (size_t)TR_MAX_SPECIES * kAT + (red_in_kt() ? 0 : red_floats());
+    return (size_t)kt_rows * kAT + dl_floats() + npad + (size_t)npad * kAT + kAT +
+           (size_t)n_ray * kAT + (red_in_kt() ? 0 : kAWarps * red_floats());
   }
 };
 
+// One CTA per (item, 64-wavenumber tile); grid (items, tiles).  Bound by instruction latency: the
+// three contractions (FP32 FMAs) are a third of the instructions, the feature sums most of the rest,
+// and a warp waits 5 to 9 cycles between two of them.  So the design is for warps in flight and
+// few instructions: the path lengths once, packed (21 KB at 100 layers instead of 43), so that
+// three CTAs share an SM (1.62 ms against 1.81 with two; 1,024 atmospheres of 100 layers, 15 tiles,
+// 5 absorbers); each absorber's corner rows alone in registers, 80 a thread, fetched one run of
+// layers ahead; eight layers' terms of two features summed by all 32 lanes at once; and loops kept
+// rolled for the instruction cache.  Before (one layer at a time, all absorbers' rows in 128
+// registers, two CTAs): 2.12 ms; 320 atmospheres of 296 tiles with CIA 15.6 ms, now 11.4.
 // RECOMP: K recomputed from the tables (a.kstore is NULL) or read from the forward's buffer;
 // instantiated separately, so each form's registers are allocated for its own K phase.
-template <int MAXMOL, bool F16, bool RECOMP>
-__global__ void __launch_bounds__(kAThreads, 2)
+template <bool F16, bool RECOMP, int CTAS>
+__global__ void __launch_bounds__(kAThreads, CTAS)
 k_adjoint_tile(AdjParams a) {
   extern __shared__ __align__(16) float smem[];
   __shared__ __align__(8) uint64_t bar;
   const FwdParams& p = a.f;
-  const int b = blockIdx.y, tile = blockIdx.x;        // tile: slot among the launched tiles
+  // items fastest: the CTAs in flight share one tile's table rows in L2 (320 atmospheres on tables
+  // of 200,000 wavenumbers: 11.4 ms against 12.1 with the tiles fastest)
+  const int b = blockIdx.x, tile = blockIdx.y;          // tile: slot among the launched tiles
   const bool jac = a.rows.n_rows > 0;
   const int wtile = jac ? a.rows.tile[tile] : tile;   // wavenumber tile
   const int jac_bin = jac ? a.rows.first_bin + a.rows.row[tile] : -1;
   const int N = p.buf.items[b].n_layers;
   if (N == 0) return;                                   // the item kernel zeroes its gradient
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const AdjSmem sp(p.max_layers, a.n_feat);
+  const int n_ray = __popc(a.ray_mask), n_zero = p.n_species - n_ray, n_act = a.n_feat - n_zero;
+  const AdjSmem sp(p.max_layers, n_act, n_ray);
   const int npad = sp.npad;
   float* Kt = smem;                                     // [max_layers][kAT]
-  float* DLT = Kt + (size_t)sp.kt_rows * kAT;           // [npad][npad], rows l, columns j
-  float* a_s = DLT + (size_t)npad * npad;               // [npad]
+  float* DLT = Kt + (size_t)sp.kt_rows * kAT;           // path lengths (AdjSmem)
+  float* a_s = DLT + sp.dl_floats();                    // [npad]
   float* Gt = a_s + npad;                               // [npad][kAT]  G_tau
   float* gd_s = Gt + (size_t)npad * kAT;                // [kAT]
-  float* ray_s = gd_s + kAT;                            // [TR_MAX_SPECIES][kAT] Rayleigh rows
-  // per warp: one layer's per-lane feature terms [n_feat][kRedPitch], summed over lanes by
-  // columns (lane f adds feature f's 32 terms in lane order); in the K tile's space when
-  // that holds them
-  float* red = (sp.red_in_kt() ? Kt : ray_s + (size_t)TR_MAX_SPECIES * kAT) +
-               (size_t)warp * a.n_feat * kRedPitch;
+  float* ray_s = gd_s + kAT;                            // [n_ray][kAT] Rayleigh rows
+  float* red = (sp.red_in_kt() ? Kt : ray_s + (size_t)n_ray * kAT) + warp * sp.red_floats();
   const int w_first = wn_first(p.wn_begin) + wtile * kAT;
 
   if (threadIdx.x == 0) { mbar_init(&bar, 1); mbar_fence_init(); }
   __syncthreads();
   if (threadIdx.x == 0) {
-    const uint32_t bytes = (uint32_t)(sizeof(float) * ((size_t)N * npad + npad));
-    mbar_arrive_expect_tx(&bar, bytes);
-    bulk_g2s(DLT, p.buf.dlt + (size_t)b * p.max_layers * npad,
-             (uint32_t)(sizeof(float) * (size_t)N * npad), &bar);
+    const uint32_t dl_bytes = (uint32_t)(sizeof(float) * (size_t)dlp_offset(N));
+    mbar_arrive_expect_tx(&bar, dl_bytes + (uint32_t)(sizeof(float) * npad));
+    bulk_g2s(DLT, p.buf.dlp + (size_t)b * dlp_offset(p.max_layers), dl_bytes, &bar);
     bulk_g2s(a_s, p.buf.aj + (size_t)b * npad, (uint32_t)(sizeof(float) * npad), &bar);
   }
-  for (int i = N * npad + threadIdx.x; i < npad * npad; i += kAThreads) DLT[i] = 0.f;
   for (int i = threadIdx.x; i < kAT; i += kAThreads) {
     const int w = w_first + i;
     float g = 0.f;
@@ -240,9 +280,11 @@ k_adjoint_tile(AdjParams a) {
     gd_s[i] = g;
   }
   if (p.ray) {                                          // the Rayleigh rows of this tile
-    for (int i = threadIdx.x; i < p.n_species * kAT; i += kAThreads) {
-      const int sp2 = i / kAT, c = i - sp2 * kAT, w = w_first + c;
-      ray_s[i] = w < p.wn_pad ? __ldg(p.ray + (size_t)sp2 * p.wn_pad + w) : 0.f;
+    for (int i = threadIdx.x; i < n_ray * kAT; i += kAThreads) {
+      const int r = i / kAT, c = i - r * kAT, w = w_first + c;
+      unsigned m = a.ray_mask;                          // its r-th species
+      for (int q = 0; q < r; ++q) m &= m - 1u;
+      ray_s[i] = w < p.wn_pad ? __ldg(p.ray + (size_t)(__ffs(m) - 1) * p.wn_pad + w) : 0.f;
     }
   }
   // ---- K tile: the forward's, or recomputed
@@ -289,7 +331,7 @@ k_adjoint_tile(AdjParams a) {
 #pragma unroll
           for (int c = 0; c < 4; ++c) us[c][0] = us[c][1] = 0.f;
 #pragma unroll
-          for (int m = 0; m < MAXMOL; ++m) {
+          for (int m = 0; m < TR_MAX_MOL; ++m) {
             if (m < p.n_mol) {
               const float xm = __ldg(ox + m);
               const size_t om = o0 + (size_t)m * p.n_p * slab_p;
@@ -336,6 +378,9 @@ k_adjoint_tile(AdjParams a) {
   }
   const bool ok = __syncthreads_and(mbar_wait_bounded(&bar, 0, p.dev_err, TR_DEVERR_TIMEOUT));
   if (!ok) { mbar_wait_bounded(&bar, 0, nullptr, 0); return; }
+  // this lane's float2 in row l of the swizzled tiles: chunk lane / 2 of 16, XORed with row / 4
+  const int lane_c = 2 * (lane & 1);
+  auto lane_col = [&](int row) { return ((((lane >> 1) ^ (row >> 2)) & (kAT / 4 - 1)) << 2) + lane_c; };
 
   const size_t item_tile = (size_t)b * a.tiles + tile;
   // ---- tau, G_tau = G_D a_j e^-tau, G_a_j = sum_v G_D (1 - e^-tau)
@@ -350,14 +395,27 @@ k_adjoint_tile(AdjParams a) {
     unsigned long long acc2[kRT / 2][2];
 #pragma unroll
     for (int r = 0; r < kRT / 2; ++r) acc2[r][0] = acc2[r][1] = 0ull;
-    for (int l = j0; l < N; ++l) {
-      const float2 kv = *reinterpret_cast<const float2*>(Kt + tix(l, 2 * lane));
-      const ulonglong2 d0 = *reinterpret_cast<const ulonglong2*>(DLT + (size_t)l * npad + j0);
-      const ulonglong2 d1 = *reinterpret_cast<const ulonglong2*>(DLT + (size_t)l * npad + j0 + 4);
+    auto tau_row = [&](const float* kr, const float* dr) {
+      const float2 kv = *reinterpret_cast<const float2*>(kr);
+      const ulonglong2 d0 = *reinterpret_cast<const ulonglong2*>(dr);
+      const ulonglong2 d1 = *reinterpret_cast<const ulonglong2*>(dr + 4);
       const unsigned long long dv[4] = {d0.x, d0.y, d1.x, d1.y};
       const unsigned long long k0 = pack_dup(kv.x), k1 = pack_dup(kv.y);
 #pragma unroll
       for (int r = 0; r < kRT / 2; ++r) { ffma2(acc2[r][0], dv[r], k0); ffma2(acc2[r][1], dv[r], k1); }
+    };
+    // four rows share the swizzle and the row length (l a multiple of 4)
+    for (int l = j0; l < N; l += 4) {
+      const float* kr = Kt + l * kAT + lane_col(l);
+      const int pitch = pad8(l + 1);
+      const float* dr = DLT + dlp_offset(l) + j0;
+      if (l + 4 <= N) {
+#pragma unroll
+        for (int u = 0; u < 4; ++u) tau_row(kr + u * kAT, dr + u * pitch);
+      } else {
+#pragma unroll 1
+        for (int u = 0; l + u < N; ++u) tau_row(kr + u * kAT, dr + u * pitch);
+      }
     }
     float acc[kRT][2];
 #pragma unroll
@@ -365,15 +423,29 @@ k_adjoint_tile(AdjParams a) {
 #pragma unroll
       for (int c = 0; c < 2; ++c)
         asm("mov.b64 {%0, %1}, %2;" : "=f"(acc[2 * r][c]), "=f"(acc[2 * r + 1][c]) : "l"(acc2[r][c]));
+    float ga[kRT];
 #pragma unroll
     for (int r = 0; r < kRT; ++r) {
       const int j = j0 + r;
       const float aj = a_s[j];
       const float e0 = __expf(-acc[r][0]), e1 = __expf(-acc[r][1]);
       *reinterpret_cast<float2*>(Gt + tix(j, 2 * lane)) = make_float2(g2.x * aj * e0, g2.y * aj * e1);
-      const float ga = warp_sum(g2.x * (1.f - e0) + g2.y * (1.f - e1));
-      if (lane == 0) a.part_a[item_tile * npad + j] = ga;
+      ga[r] = g2.x * (1.f - e0) + g2.y * (1.f - e1);
     }
+    // the eight rays' sums over the warp, halving the rays as the lanes pair up (16, 8, 4 apart,
+    // then 2 and 1): lane 4r ends with the sum of ray r
+#pragma unroll
+    for (int o = 16, n = kRT / 2; o >= 4; o >>= 1, n >>= 1) {
+      const bool up = lane & o;
+#pragma unroll
+      for (int r = 0; r < n; ++r) {
+        const float mine = up ? ga[r + n] : ga[r], other = up ? ga[r] : ga[r + n];
+        ga[r] = mine + __shfl_xor_sync(0xffffffffu, other, o);
+      }
+    }
+    ga[0] += __shfl_xor_sync(0xffffffffu, ga[0], 2);
+    ga[0] += __shfl_xor_sync(0xffffffffu, ga[0], 1);
+    if (!(lane & 3)) a.part_a[item_tile * npad + j0 + (lane >> 2)] = ga[0];
   }
   for (int j = N + threadIdx.x; j < npad; j += kAThreads) {
     for (int c = 0; c < kAT; ++c) Gt[(size_t)j * kAT + c] = 0.f;
@@ -400,6 +472,7 @@ k_adjoint_tile(AdjParams a) {
       unsigned long long acc2[4][4];
 #pragma unroll
       for (int x = 0; x < 4; ++x) acc2[x][0] = acc2[x][1] = acc2[x][2] = acc2[x][3] = 0ull;
+#pragma unroll 2
       for (int c = 0; c < kAT; c += 4) {
         ulonglong2 g[4], k[4];
 #pragma unroll
@@ -416,23 +489,38 @@ k_adjoint_tile(AdjParams a) {
             ffma2(acc2[x][y], g[x].y, k[y].y);
           }
       }
+      // whole 16-byte rows: the entries with l < j or l >= N are not read
 #pragma unroll
-      for (int x = 0; x < 4; ++x)
+      for (int x = 0; x < 4; ++x) {
+        float v[4];
 #pragma unroll
         for (int y = 0; y < 4; ++y) {
-          const int j = j0 + x, l = l0 + y;
-          float e0, e1;
-          asm("mov.b64 {%0, %1}, %2;" : "=f"(e0), "=f"(e1) : "l"(acc2[x][y]));
-          if (j <= l && l < N) pdl[(size_t)j * npad + l] = e0 + e1;
+          const float2 e = unpack2(acc2[x][y]);
+          v[y] = j0 + x <= l0 + y && l0 + y < N ? e.x + e.y : 0.f;
         }
+        if (j0 + x < N)
+          *reinterpret_cast<float4*>(pdl + (size_t)(j0 + x) * npad + l0) = make_float4(v[0], v[1], v[2], v[3]);
+      }
     }
   }
 
   // ---- G_K_l(v) = sum_{j<=l} DL[j][l] G_tau_j(v) over 8-layer tiles, then per-layer sums
-  if (sp.red_in_kt()) __syncthreads();                 // every warp is done reading K
+  if (sp.red_in_kt()) __syncthreads();                  // every warp is done reading K
   const int n_lt = (N + kRT - 1) / kRT;
-  const int nm = p.n_mol, ns = p.ray ? p.n_species : 0, nq = p.n_cia;
-  const int f_dS = nm, f_R = 2 * nm, f_C = 2 * nm + p.n_species, f_dC = f_C + nq, f_K = f_dC + nq;
+  const int nm = p.n_mol, nq = p.n_cia;
+  // columns of the sums: the features without the species that have no Rayleigh cross-sections,
+  // whose sums are zero
+  const int f_dS = nm, f_R = 2 * nm, f_C = 2 * nm + n_ray, f_dC = f_C + nq, f_K = f_dC + nq;
+  auto column_of = [&](int f) -> int {                  // feature f's column, or -1: zero
+    if (f < 2 * nm) return f;
+    const int sp_i = f - 2 * nm;
+    if (sp_i >= p.n_species) return f - n_zero;
+    return (a.ray_mask >> sp_i) & 1u ? f_R + __popc(a.ray_mask & ((1u << sp_i) - 1u)) : -1;
+  };
+  float* hd = red + kRedRows * kRedPitch;               // [kRT][kHdr]
+  float* sums = hd + kHdr * kRT;                        // [kRT][n_act]
+  const size_t slab_t = (size_t)p.wn_pad, slab_p = (size_t)p.n_t * p.wn_pad;
+  const int wq = in_row ? w2 : 0;
   // a tile's cost grows with its layer index (the contraction runs over j <= l), so the warps
   // take the tiles from the top down, in a snake over the warps: the largest tiles first, then
   // the smallest ones to the warps that took the smaller of the large ones
@@ -441,146 +529,182 @@ k_adjoint_tile(AdjParams a) {
     const int kt = round * kAWarps + pos;
     if (kt >= n_lt) break;
     const int lt = n_lt - 1 - kt;
-    const int l0 = lt * kRT;
-    // the tile's layer headers, lane r < kRT holding layer l0 + r's (brackets, weights, flags
-    // and reciprocal T spacings), loaded before the contraction so that their latency
-    // overlaps it; each layer below takes them by shuffle
-    int4 hb = make_int4(0, 0, 0, 0);
-    float4 hw = make_float4(0.f, 0.f, 0.f, 0.f);
-    unsigned hfl = 0u;
-    float hidt = 0.f, hidc = 0.f;
-    if (lane < kRT && l0 + lane < N) {
+    const int l0 = lt * kRT, nr = min(kRT, N - l0);
+    // the tile's layer headers (brackets, weights and reciprocal T spacings), lane r holding
+    // layer l0 + r's: loaded before the contraction so that their latency overlaps it
+    int cell = 0, itc = 0;
+    float tp = 0.f, tt = 0.f, ttc = 0.f, idt = 0.f, idc = 0.f;
+    if (lane < nr) {
       const int4* dd = reinterpret_cast<const int4*>(LD + l0 + lane);
-      hb = __ldg(dd);                                    // ip, it, itc
-      hw = as_float4(__ldg(dd + 1));               // rho, tp, tt, ttc
-      hfl = d_flags(__ldg(dd + 2));
-      hidt = (hfl & kLayerTClamp) ? 0.f : (float)a.inv_dt[hb.y];
-      hidc = (nq > 0 && !(hfl & kLayerTcClamp)) ? (float)a.inv_dtc[hb.z] : 0.f;
+      const int4 hb = __ldg(dd);                         // ip, it, itc
+      const float4 hw = as_float4(__ldg(dd + 1));        // rho, tp, tt, ttc
+      const unsigned fl = d_flags(__ldg(dd + 2));
+      cell = hb.x * p.n_t + hb.y; itc = hb.z;
+      tp = hw.y; tt = hw.z; ttc = hw.w;
+      idt = (fl & kLayerTClamp) ? 0.f : (float)a.inv_dt[hb.y];
+      idc = (nq > 0 && !(fl & kLayerTcClamp)) ? (float)a.inv_dtc[hb.z] : 0.f;
     }
     float acc[kRT][2];
-    const int jmax = min(N, l0 + kRT);
-    if constexpr (MAXMOL <= 5) {
-      // packed FP32 pairs over layers: acc2[r][c] holds layers (2r, 2r+1) at wavenumber c (with
-      // eight absorbers the extra registers spill, so that form keeps scalar FMAs)
-      unsigned long long acc2[kRT / 2][2];
-#pragma unroll
-      for (int r = 0; r < kRT / 2; ++r) acc2[r][0] = acc2[r][1] = 0ull;
-      for (int j = 0; j < jmax; ++j) {
-        const float2 g = *reinterpret_cast<const float2*>(Gt + tix(j, 2 * lane));
-        const unsigned long long gx = pack_dup(g.x), gy = pack_dup(g.y);
-#pragma unroll
-        for (int r = 0; r < kRT / 2; ++r) {
-          // zero for j > l and rows >= N
-          const unsigned long long dl = pack2(DLT[(size_t)(l0 + 2 * r) * npad + j],
-                                              DLT[(size_t)(l0 + 2 * r + 1) * npad + j]);
-          ffma2(acc2[r][0], dl, gx);
-          ffma2(acc2[r][1], dl, gy);
-        }
-      }
-#pragma unroll
-      for (int r = 0; r < kRT / 2; ++r)
-#pragma unroll
-        for (int c = 0; c < 2; ++c) {
-          const float2 v = unpack2(acc2[r][c]);
-          acc[2 * r][c] = v.x;
-          acc[2 * r + 1][c] = v.y;
-        }
-    } else {
+    {
 #pragma unroll
       for (int r = 0; r < kRT; ++r) acc[r][0] = acc[r][1] = 0.f;
-      for (int j = 0; j < jmax; ++j) {
-        const float2 g = *reinterpret_cast<const float2*>(Gt + tix(j, 2 * lane));
+      // rows l0 .. l0 + 7 of the packed path lengths have one length; four rays at a time (one
+      // 16-byte load a row; they share the swizzle).  Rays beyond N: both factors are zero
+      const int pitch = l0 + kRT;
+      const float* dr = DLT + dlp_offset(l0);
+      const int jmax = min(N, l0 + kRT);
+      for (int j = 0; j < jmax; j += 4) {
+        float4 d[kRT];
 #pragma unroll
-        for (int r = 0; r < kRT; ++r) {
-          const float dl = DLT[(size_t)(l0 + r) * npad + j];   // zero for j > l and rows >= N
-          acc[r][0] = fmaf(dl, g.x, acc[r][0]);
-          acc[r][1] = fmaf(dl, g.y, acc[r][1]);
-        }
-      }
-    }
-    // the corner rows of the current (P, T) cell at this lane's two wavenumbers: consecutive
-    // layers of one cell (a segment) share them, so they are gathered from L2 once per
-    // segment, all together, instead of once per layer
-    unsigned long long cs[MAXMOL][4];                  // (sigma(v), sigma(v + 1)) pairs
-    int c_ip = -1, c_it = -1;
-    for (int r = 0; r < kRT; ++r) {
-      const int l = l0 + r;
-      if (l >= N) break;
-      float* pf = a.part_f + (item_tile * p.max_layers + l) * a.n_feat;
-      const float gk0 = in_row ? acc[r][0] : 0.f, gk1 = in_row ? acc[r][1] : 0.f;
-      const int d_ip = __shfl_sync(0xffffffffu, hb.x, r), d_it = __shfl_sync(0xffffffffu, hb.y, r);
-      const int d_itc = __shfl_sync(0xffffffffu, hb.z, r);
-      const float tp = __shfl_sync(0xffffffffu, hw.y, r), tt = __shfl_sync(0xffffffffu, hw.z, r);
-      const float ttc = __shfl_sync(0xffffffffu, hw.w, r);
-      const float idt = __shfl_sync(0xffffffffu, hidt, r);
-      const float idc = __shfl_sync(0xffffffffu, hidc, r);
-      const size_t slab_t = (size_t)p.wn_pad, slab_p = (size_t)p.n_t * p.wn_pad;
-      const int wq = in_row ? w2 : 0;
-      if (d_ip != c_ip || d_it != c_it) {               // a new cell (warp-uniform)
-        const size_t o0 = ((size_t)d_ip * p.n_t + d_it) * p.wn_pad + wq;
+        for (int r = 0; r < kRT; ++r) d[r] = *reinterpret_cast<const float4*>(dr + r * pitch + j);
+        const float* gr = Gt + j * kAT + lane_col(j);
 #pragma unroll
-        for (int m = 0; m < MAXMOL; ++m) {
-          if (m < nm) {
-            const size_t om = o0 + (size_t)m * p.n_p * slab_p;
-            const float2 v0 = sig2<F16>(p, m, om), v1 = sig2<F16>(p, m, om + slab_t),
-                         v2 = sig2<F16>(p, m, om + slab_p), v3 = sig2<F16>(p, m, om + slab_p + slab_t);
-            cs[m][0] = pack2(v0.x, v0.y);
-            cs[m][1] = pack2(v1.x, v1.y);
-            cs[m][2] = pack2(v2.x, v2.y);
-            cs[m][3] = pack2(v3.x, v3.y);
+        for (int u = 0; u < 4; ++u) {
+          const float2 g = *reinterpret_cast<const float2*>(gr + u * kAT);
+#pragma unroll
+          for (int r = 0; r < kRT; ++r) {
+            const float dl = u == 0 ? d[r].x : u == 1 ? d[r].y : u == 2 ? d[r].z : d[r].w;
+            acc[r][0] = fmaf(dl, g.x, acc[r][0]);
+            acc[r][1] = fmaf(dl, g.y, acc[r][1]);
           }
         }
-        c_ip = d_ip; c_it = d_it;
       }
-      // this lane's terms of every feature of layer l (its two wavenumbers, as packed pairs)
-      const unsigned long long tt2 = pack_dup(tt), tp2 = pack_dup(tp), up2 = pack_dup(1.f - tp);
-      const unsigned long long idt2 = pack_dup(idt);
-#pragma unroll
-      for (int m = 0; m < MAXMOL; ++m) {
-        if (m < nm) {
-          // sigma(T) at both pressures, then sigma(P); d sigma / dT of the same bracket
-          const unsigned long long d0 = sub2(cs[m][1], cs[m][0]), d1 = sub2(cs[m][3], cs[m][2]);
-          const unsigned long long a1 = fma2(d0, tt2, cs[m][0]), a2 = fma2(d1, tt2, cs[m][2]);
-          const float2 sg = unpack2(fma2(sub2(a2, a1), tp2, a1));
-          const float2 dt = unpack2(mul2(fma2(d0, up2, mul2(d1, tp2)), idt2));
-          red[m * kRedPitch + lane] = fmaf(gk0, sg.x, gk1 * sg.y);
-          red[(f_dS + m) * kRedPitch + lane] = fmaf(gk0, dt.x, gk1 * dt.y);
-        }
-      }
-      for (int s = 0; s < p.n_species; ++s) {
-        float fr = 0.f;
-        if (s < ns) {
-          const float2 v = *reinterpret_cast<const float2*>(ray_s + s * kAT + 2 * lane);
-          fr = gk0 * v.x + gk1 * v.y;
-        }
-        red[(f_R + s) * kRedPitch + lane] = fr;
-      }
-      if (nq > 0) {
-        for (int q = 0; q < nq; ++q) {
-          const float* bq = p.cia + ((size_t)q * p.n_t_cia + d_itc) * p.wn_pad + wq;
-          const float2 c0 = ldg2(bq), c1 = ldg2(bq + p.wn_pad);
-          const float sg0 = c0.x + (c1.x - c0.x) * ttc, sg1 = c0.y + (c1.y - c0.y) * ttc;
-          red[(f_C + q) * kRedPitch + lane] = gk0 * sg0 + gk1 * sg1;
-          red[(f_dC + q) * kRedPitch + lane] = gk0 * (c1.x - c0.x) * idc + gk1 * (c1.y - c0.y) * idc;
-        }
-      }
-      red[f_K * kRedPitch + lane] = gk0 + gk1;
-      __syncwarp();
-      for (int f = lane; f < a.n_feat; f += 32) {       // feature f: its 32 terms in lane order
-        const float4* row = reinterpret_cast<const float4*>(red + f * kRedPitch);
-        // four chains (terms k = 0, 1, 2, 3 mod 4) as two packed pairs, fixed order
-        unsigned long long s01 = 0ull, s23 = 0ull;
-#pragma unroll
-        for (int k = 0; k < 8; ++k) {
-          const float4 v = row[k];
-          s01 = add2(s01, pack2(v.x, v.y));
-          s23 = add2(s23, pack2(v.z, v.w));
-        }
-        const float2 u = unpack2(s01), w = unpack2(s23);
-        pf[f] = (u.x + u.y) + (w.x + w.y);
-      }
-      __syncwarp();                                     // red is free for the next layer
     }
+    if (!in_row) {
+#pragma unroll
+      for (int r = 0; r < kRT; ++r) acc[r][0] = acc[r][1] = 0.f;
+    }
+    // layers where the (P, T) cell and the CIA bracket change: runs of layers share their rows
+    const int cell_b = __shfl_up_sync(0xffffffffu, cell, 1), itc_b = __shfl_up_sync(0xffffffffu, itc, 1);
+    const unsigned chg = __ballot_sync(0xffffffffu, lane < nr && (lane == 0 || cell != cell_b));
+    const unsigned chc = __ballot_sync(0xffffffffu, lane < nr && (lane == 0 || itc != itc_b));
+    if (lane < nr) {
+      float* h = hd + kHdr * lane;
+      *reinterpret_cast<float4*>(h) = make_float4(tt, tt, tp, tp);
+      *reinterpret_cast<float4*>(h + 4) = make_float4(idt, idt, __int_as_float(cell), __int_as_float(itc));
+      *reinterpret_cast<float2*>(h + 8) = make_float2(ttc, idc);
+    }
+    __syncwarp();
+    // the sums of columns fa and fb (rows 2r and 2r + 1 hold layer r's terms of each): lanes 2i
+    // and 2i + 1 add row i's terms 0, 1 and 2, 3 mod 4 as chains in lane order
+    auto reduce = [&](int fa, int fb) {
+      __syncwarp();
+      const unsigned long long* row = reinterpret_cast<const unsigned long long*>(
+          red + (lane >> 1) * kRedPitch + 2 * (lane & 1));
+      unsigned long long t = 0ull;
+#pragma unroll
+      for (int k = 0; k < 8; ++k) t = add2(t, row[2 * k]);
+      const float2 u = unpack2(t);
+      float v = u.x + u.y;
+      v += __shfl_xor_sync(0xffffffffu, v, 1);
+      const int f = lane & 2 ? fb : fa;
+      if (!(lane & 1) && f >= 0) sums[(lane >> 2) * n_act + f] = v;
+      __syncwarp();                                      // the rows are free again
+    };
+    // absorbers, one at a time: the rows of the next run's (or the next absorber's first) cell
+    // are fetched while a run's layers are done
+    SigRaw<F16> nx[4];
+    auto fetch = [&](int m, int r) {
+      const size_t o = ((size_t)m * p.n_p * p.n_t + __float_as_int(hd[kHdr * r + 6])) * slab_t + wq;
+      nx[0] = sig_fetch<F16>(p, o);
+      nx[1] = sig_fetch<F16>(p, o + slab_t);
+      nx[2] = sig_fetch<F16>(p, o + slab_p);
+      nx[3] = sig_fetch<F16>(p, o + slab_p + slab_t);
+    };
+    if (nm > 0) fetch(0, 0);
+    const unsigned long long one2 = pack_dup(1.f);
+    // The layers four at a time in a loop: unrolled over all eight, the kernel's code outgrew the
+    // instruction cache (26% of the issue slots were lost to it).
+    for (int m = 0; m < nm; ++m) {
+      const float c = F16 ? p.logsig_off[m] : 0.f;
+      // of the current cell, (v, v + 1) pairs: sigma at the lower T and its step to the upper, at
+      // the lower and the upper pressure
+      unsigned long long s0 = 0ull, d0 = 0ull, s1 = 0ull, d1 = 0ull;
+#pragma unroll 1
+      for (int rh = 0; rh < kRT; rh += kRT / 2) {
+#pragma unroll
+        for (int q = 0; q < kRT / 2; ++q) {
+          const int r = rh + q;
+          if (r >= nr) break;
+          const float gk0 = rh ? acc[q + kRT / 2][0] : acc[q][0], gk1 = rh ? acc[q + kRT / 2][1] : acc[q][1];
+          if ((chg >> r) & 1u) {
+            s0 = sig_value<F16>(nx[0], c);
+            d0 = sub2(sig_value<F16>(nx[1], c), s0);
+            s1 = sig_value<F16>(nx[2], c);
+            d1 = sub2(sig_value<F16>(nx[3], c), s1);
+            const unsigned later = chg & ~((2u << r) - 1u);
+            const int mn = later ? m : m + 1;
+            if (mn < nm) fetch(mn, later ? __ffs(later) - 1 : 0);
+          }
+          const float* h = hd + kHdr * r;
+          const ulonglong2 t = *reinterpret_cast<const ulonglong2*>(h);          // (tt, tt), (tp, tp)
+          const unsigned long long idt2 = *reinterpret_cast<const unsigned long long*>(h + 4);
+          // sigma(T) at both pressures, then sigma(P); d sigma / dT of the same bracket
+          const unsigned long long a1 = fma2(d0, t.x, s0), a2 = fma2(d1, t.x, s1);
+          const float2 sg = unpack2(fma2(sub2(a2, a1), t.y, a1));
+          const float2 dt = unpack2(mul2(fma2(d0, sub2(one2, t.y), mul2(d1, t.y)), idt2));
+          red[2 * r * kRedPitch + lane] = fmaf(gk0, sg.x, gk1 * sg.y);
+          red[(2 * r + 1) * kRedPitch + lane] = fmaf(gk0, dt.x, gk1 * dt.y);
+        }
+      }
+      reduce(m, f_dS + m);
+    }
+    if (nq > 0) {
+      // CIA pairs alike: two rows of the bracket
+      float2 nc[2];
+      auto fetch_c = [&](int q, int r) {
+        const float* bq = p.cia + ((size_t)q * p.n_t_cia + __float_as_int(hd[kHdr * r + 7])) * p.wn_pad + wq;
+        nc[0] = ldg2(bq);
+        nc[1] = ldg2(bq + p.wn_pad);
+      };
+      fetch_c(0, 0);
+#pragma unroll 1
+      for (int q = 0; q < nq; ++q) {
+        float2 c0 = make_float2(0.f, 0.f), c1 = c0;
+#pragma unroll 1
+        for (int rh = 0; rh < kRT; rh += kRT / 2) {
+#pragma unroll
+          for (int i = 0; i < kRT / 2; ++i) {
+            const int r = rh + i;
+            if (r >= nr) break;
+            const float gk0 = rh ? acc[i + kRT / 2][0] : acc[i][0], gk1 = rh ? acc[i + kRT / 2][1] : acc[i][1];
+            if ((chc >> r) & 1u) {
+              c0 = nc[0]; c1 = nc[1];
+              const unsigned later = chc & ~((2u << r) - 1u);
+              const int qn = later ? q : q + 1;
+              if (qn < nq) fetch_c(qn, later ? __ffs(later) - 1 : 0);
+            }
+            const float2 h = *reinterpret_cast<const float2*>(hd + kHdr * r + 8);   // ttc, 1/dTc
+            const float sg0 = c0.x + (c1.x - c0.x) * h.x, sg1 = c0.y + (c1.y - c0.y) * h.x;
+            red[2 * r * kRedPitch + lane] = gk0 * sg0 + gk1 * sg1;
+            red[(2 * r + 1) * kRedPitch + lane] = gk0 * (c1.x - c0.x) * h.y + gk1 * (c1.y - c0.y) * h.y;
+          }
+        }
+        reduce(f_C + q, f_dC + q);
+      }
+    }
+    // Rayleigh species and, last, the plain sum
+#pragma unroll 1
+    for (int i = 0; i <= n_ray; i += 2) {
+#pragma unroll 1
+      for (int h = 0; h < 2; ++h) {
+        if (i + h < n_ray) {
+          const float2 v = *reinterpret_cast<const float2*>(ray_s + (i + h) * kAT + 2 * lane);
+#pragma unroll
+          for (int r = 0; r < kRT; ++r) red[(2 * r + h) * kRedPitch + lane] = acc[r][0] * v.x + acc[r][1] * v.y;
+        } else if (i + h == n_ray) {
+#pragma unroll
+          for (int r = 0; r < kRT; ++r) red[(2 * r + h) * kRedPitch + lane] = acc[r][0] + acc[r][1];
+        }
+      }
+      reduce(i < n_ray ? f_R + i : f_K, i + 1 < n_ray ? f_R + i + 1 : i + 1 == n_ray ? f_K : -1);
+    }
+    float* pf = a.part_f + (item_tile * p.max_layers + l0) * a.n_feat;
+    for (int f = lane; f < a.n_feat; f += 32) {
+      const int col = column_of(f);
+      for (int r = 0; r < nr; ++r) pf[r * a.n_feat + f] = col >= 0 ? sums[r * n_act + col] : 0.f;
+    }
+    __syncwarp();                                        // headers and sums are free for the next tile
   }
 }
 
@@ -1114,15 +1238,16 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   ap.kstore = use_kstore ? kbuf : nullptr;
   ap.kcols = forward_kcols(bins->dev.i0, n_in);
   ap.t_ptr = bins->dev.t_ptr; ap.t_bin = bins->dev.t_bin; ap.t_w = bins->dev.t_w;
-  const size_t smem = sizeof(float) * AdjSmem(d->max_layers, n_feat).floats();
-  static_assert(TR_MAX_MOL == 8, "adjoint instantiated for up to 5 or 8 molecules");
-  void (*kern)(AdjParams);
-  if (t->n_mol <= 5)
-    kern = mixed ? (use_kstore ? k_adjoint_tile<5, true, false> : k_adjoint_tile<5, true, true>)
-                 : (use_kstore ? k_adjoint_tile<5, false, false> : k_adjoint_tile<5, false, true>);
-  else
-    kern = mixed ? (use_kstore ? k_adjoint_tile<8, true, false> : k_adjoint_tile<8, true, true>)
-                 : (use_kstore ? k_adjoint_tile<8, false, false> : k_adjoint_tile<8, false, true>);
+  ap.ray_mask = t->has_ray ? t->ray_mask : 0u;
+  const int n_ray = __builtin_popcount(ap.ray_mask), n_act = n_feat - (t->n_species - n_ray);
+  const size_t smem = sizeof(float) * AdjSmem(d->max_layers, n_act, n_ray).floats();
+  // three CTAs per SM (80 registers a thread) where their shared memory fits: 1.62 ms against 1.81
+  // (k_adjoint_tile)
+  const bool three = smem <= kThreeCtaSmem;
+  void (*kern)(AdjParams) =
+      use_kstore ? (mixed ? (three ? k_adjoint_tile<true, false, 3> : k_adjoint_tile<true, false, 2>)
+                          : (three ? k_adjoint_tile<false, false, 3> : k_adjoint_tile<false, false, 2>))
+                 : (mixed ? k_adjoint_tile<true, true, 2> : k_adjoint_tile<false, true, 2>);
   err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
   if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint tile kernel: ") + cudaGetErrorString(err));
   int dev = 0, n_sm = 0;
@@ -1145,7 +1270,7 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
     ap.rows = rows; ap.tiles = slots;
     {
       KernelTimer kt(ctx, "k_adjoint_tile", s);
-      kern<<<dim3(slots, bc), kAThreads, smem, s>>>(ap);
+      kern<<<dim3(bc, slots), kAThreads, smem, s>>>(ap);
       err = cudaGetLastError();
     }
     if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint tile kernel: ") + cudaGetErrorString(err));

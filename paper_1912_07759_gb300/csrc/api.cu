@@ -596,7 +596,10 @@ extern "C" int tr_load_xsec_tables(tr_ctx* ctx, const tr_table_desc* d, tr_table
       const double* src = d->rayleigh + (size_t)s * W;
       const int ex = scale_exponent(src, W);
       t->ray_scale[s] = std::ldexp(1.0, ex);
-      for (size_t i = 0; i < W; ++i) tmp[(size_t)s * WP + i] = (float)std::ldexp(src[i], -ex);
+      for (size_t i = 0; i < W; ++i) {
+        tmp[(size_t)s * WP + i] = (float)std::ldexp(src[i], -ex);
+        if (src[i] != 0.0) t->ray_mask |= 1u << s;
+      }
     }
     e = cudaMalloc(&t->d_ray, sizeof(float) * tmp.size()); if (e) return bail("alloc rayleigh");
     e = cudaMemcpy(t->d_ray, tmp.data(), sizeof(float) * tmp.size(), cudaMemcpyHostToDevice);

@@ -471,6 +471,7 @@ struct tr_tables {
   int n_cia = 0, n_t_cia = 0, n_species = 0, storage = 0, oor_mode = 0;
   int interp_mode = 0;                     // TR_INTERP_*
   int has_ray = 0;
+  unsigned ray_mask = 0;                   // species whose Rayleigh row has a non-zero value
   int cia_a[TR_MAX_CIA] = {}, cia_b[TR_MAX_CIA] = {};
   double cia_scale[TR_MAX_CIA] = {};
   double ray_scale[TR_MAX_SPECIES] = {};
