@@ -1188,8 +1188,11 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   const size_t db = al256(dl_tile_bytes(B, d->max_layers, precision));
   const size_t need = fwd + kb + db + adjoint_extra_bytes(t, d, bins, B);
   ItemBuffers buf; double* depth = nullptr; char* extra = nullptr;
+  // the altitudes and path lengths on a second branch beside the first opacity kernel
+  Fork fk;
+  Fork* fork = fork_ready(ctx, &fk) ? &fk : nullptr;
   int rc = prepare_batch(ctx, t, d, n_in, need, B, d_theta, d_nlayers, d_status, ws, ws_bytes,
-                         s, &buf, &depth, &extra);
+                         s, &buf, &depth, &extra, fork);
   if (rc != TR_OK) return rc;
   float* kbuf = reinterpret_cast<float*>(extra);
   void* dl16 = db > 0 ? extra + kb : nullptr;
@@ -1306,8 +1309,12 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
     double* bin_out = binned + (size_t)b0 * bins->dev.n_bin;
     if (need_binned || use_kstore) {
       rc = run_forward(ctx, t, d->max_layers, rb, bc, bins->dev.i0, n_in, out, n_in, precision, s,
-                       kbuf, dl16, &fc, /*opacity_only=*/!need_binned);
+                       kbuf, dl16, &fc, /*opacity_only=*/!need_binned, fork);
+      join_fork(ctx, fork, s);
       if (rc != TR_OK) return rc;
+    } else {
+      err = fork_start(ctx, fork, s, false);
+      if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
     }
     if (need_binned) {
       KernelTimer kt(ctx, "k_bin", s);

@@ -303,7 +303,7 @@ cudaError_t tr::fork_start(tr_ctx* ctx, Fork* f, cudaStream_t s, bool detached) 
   {
     KernelTimer kt(ctx, "k_altitude", ps);
     const cudaError_t e = launch_altitude(f->gp, f->B, f->buf, ps);
-    if (e != cudaSuccess) return e;
+    if (e != cudaSuccess || !f->pathlen) return e;
   }
   KernelTimer kt(ctx, "k_pathlen", ps);
   return launch_pathlen(f->gp, f->B, f->buf, ps);
@@ -955,7 +955,7 @@ int tr::run_forward(tr_ctx* ctx, const tr_tables* t, int max_layers, const ItemB
     return launch_dl_tf32(buf, B, max_layers, dl16, st);
   };
   // with a pending branch they follow the path lengths there, after the first opacity launch
-  const bool branch = fork && fork->pending && !opacity_only;
+  const bool branch = fork && fork->pending;
   if (!branch) {
     e = fork_start(ctx, fork, s, false);
     if (e == cudaSuccess) e = tiles_kernel(s);
@@ -978,7 +978,7 @@ int tr::run_forward(tr_ctx* ctx, const tr_tables* t, int max_layers, const ItemB
         KernelTimer kt(ctx, mixed ? "k_opacity_fp16" : "k_opacity_fp32", s);
         e = launch_opacity(p, t, bc, kbuf, choice ? choice->per_sm : 0, s);
       }
-      if (e != cudaSuccess || opacity_only) break;
+      if (e != cudaSuccess) break;
       if (branch && first) {
         // the path lengths and their tiles beside the opacity kernel, then the join
         e = fork_start(ctx, fork, s, true);
@@ -986,6 +986,7 @@ int tr::run_forward(tr_ctx* ctx, const tr_tables* t, int max_layers, const ItemB
         join_fork(ctx, fork, s);
         if (e != cudaSuccess) break;
       }
+      if (opacity_only) break;
       first = false;
       KernelTimer kt(ctx, mixed ? "k_contract_umma" : kind == kContractTC ? "k_contract_tc"
                                                                           : "k_contract_fp32", s);

@@ -173,10 +173,12 @@ int check_emission_args(tr_ctx* ctx, int n_mu, double t_star) {
 }
 
 // Opacity (two-stage opacity kernel, chunk by chunk through kbuf) then the emission pass, for
-// items [0, B) of `buf`, native range [wn_begin, wn_begin + wn_count).
+// items [0, B) of `buf`, native range [wn_begin, wn_begin + wn_count).  fork: a pending altitude
+// kernel, run beside the first opacity launch (one model of 200,000 wavenumbers: 142 us a call with altitudes
+// and path lengths before it, 125 so).
 int run_emission(tr_ctx* ctx, const tr_tables* t, int max_layers, const ItemBuffers& buf, int B,
                  int wn_begin, int wn_count, double* out, long long stride, int precision,
-                 float* kbuf, int n_mu, double t_star, cudaStream_t s) {
+                 float* kbuf, int n_mu, double t_star, cudaStream_t s, Fork* fork = nullptr) {
   const bool mixed = precision == TR_PREC_MIXED;
   if (precision != TR_PREC_FP32 && !mixed) return set_error(ctx, TR_ERR_ARG, "unknown precision");
   if (!mixed && !t->d_sigma && t->n_mol > 0)
@@ -213,6 +215,10 @@ int run_emission(tr_ctx* ctx, const tr_tables* t, int max_layers, const ItemBuff
     {
       KernelTimer kt(ctx, mixed ? "k_opacity_fp16" : "k_opacity_fp32", s);
       e = launch_opacity(fp, t, bc, kbuf, 0, s);
+    }
+    if (e == cudaSuccess && b0 == 0) {
+      e = fork_start(ctx, fork, s, true);
+      join_fork(ctx, fork, s);
     }
     if (e != cudaSuccess) break;
     ep.b_off = b0;
@@ -274,18 +280,21 @@ extern "C" int tr_forward_emission_batch(tr_ctx* ctx, const tr_tables* t,
   const int n_in = d_native ? 0 : bins->dev.i1 - bins->dev.i0;
   const size_t need = forward_batch_need(t, d, B, bins, d_native != nullptr, precision);
   ItemBuffers buf; double* depth = nullptr; char* extra = nullptr;
+  Fork fk;
+  fk.pathlen = false;
+  Fork* fork = fork_ready(ctx, &fk) ? &fk : nullptr;
   rc = prepare_batch(ctx, t, d, n_in, need, B, d_theta, d_nlayers, d_status, ws, ws_bytes, s,
-                     &buf, &depth, &extra);
+                     &buf, &depth, &extra, fork);
   if (rc != TR_OK) return rc;
   float* kbuf = reinterpret_cast<float*>(extra);
   if (d_native) {
     rc = run_emission(ctx, t, d->max_layers, buf, B, 0, t->n_wn, d_native, t->n_wn, precision,
-                      kbuf, n_mu, t_star, s);
+                      kbuf, n_mu, t_star, s, fork);
     if (rc != TR_OK || !d_binned) return rc;
     return run_bin(ctx, bins, B, d_native, t->n_wn, 0, d_binned, s);
   }
   rc = run_emission(ctx, t, d->max_layers, buf, B, bins->dev.i0, n_in, depth, n_in, precision,
-                    kbuf, n_mu, t_star, s);
+                    kbuf, n_mu, t_star, s, fork);
   if (rc != TR_OK) return rc;
   return run_bin(ctx, bins, B, depth, n_in, bins->dev.i0, d_binned, s);
 }

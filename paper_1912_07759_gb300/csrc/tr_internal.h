@@ -345,8 +345,8 @@ cudaError_t launch_contract_umma(const FwdParams& p, int Bc, const float* kbuf, 
                                  cudaStream_t s);
 // adjoint.cu: extra workspace of the adjoint
 size_t adjoint_extra_bytes(const tr_tables* t, const tr_batch_desc* d, const tr_bins* bins, int B);
-// The batched forward's second branch: the path-length kernels (which only the contraction
-// reads) run on the context's auxiliary stream beside the opacity kernel.  prepare_batch
+// The batched calls' second branch: the altitude and path-length kernels (which only the kernels
+// after the opacity read) run on the context's auxiliary stream beside the opacity kernel.  prepare_batch
 // records the fork event after the profile kernel and leaves the path-length kernel pending;
 // run_forward issues it (and the path-length tile kernel) on the auxiliary stream, which
 // waits for the fork event, right after the first opacity launch, and joins before the first
@@ -357,6 +357,7 @@ size_t adjoint_extra_bytes(const tr_tables* t, const tr_batch_desc* d, const tr_
 struct Fork {
   cudaStream_t aux = nullptr;
   bool open = false, pending = false;
+  bool pathlen = true;      // false: the altitudes alone (emission reads no path lengths)
   GeomParams gp{};
   int B = 0;
   ItemBuffers buf{};
