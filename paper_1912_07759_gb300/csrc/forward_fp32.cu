@@ -351,9 +351,9 @@ cudaError_t launch_opacity_p(const FwdParams& p, const CUtensorMap& sig, const C
 
 // ---- FP32 contraction + depth, persistent (second stage of the two-stage form)
 //
-// Work unit = one item x kTW wavenumbers of K; the units are split into contiguous ranges, one
-// per CTA (item-major, so consecutive units of a CTA mostly share the item and its path
-// lengths).  A producer warp loads each unit's K tile [N][kTW] by 2-D TMA boxes of kCB rows
+// Work unit = one item x kTW wavenumbers of K; the units are split into contiguous ranges of about
+// equal cost, one per CTA (item-major, so consecutive units of a CTA mostly share the item and its
+// path lengths; a unit's cost grows with the square of its item's layer count).  A producer warp loads each unit's K tile [N][kTW] by 2-D TMA boxes of kCB rows
 // into one of up to three tile slots, plus the item's packed path lengths and annulus weights by
 // bulk copy when the item changes (after every earlier unit is done with them), on a barrier of
 // their own: a K tile of the item's second unit can land before them.  The W
@@ -390,6 +390,62 @@ __device__ __forceinline__ bool wait_slot(const int* slot_unit, int k, const int
   return false;
 }
 
+// Cost of a unit of an item of N layers, in rows of a 16-ray tile: its tiles' rows, and the
+// exponentials and the hand-over of each tile, about eight rows' worth.
+__device__ __forceinline__ unsigned unit_cost(int N) {
+  const int n_rt = (N + kRT - 1) / kRT;
+  return (unsigned)(n_rt * N - kRT / 2 * n_rt * (n_rt - 1) + 8 * n_rt + 4);
+}
+
+// This CTA's units [x, y): unit u belongs to CTA g when its cost offset lies in [g, g + 1) / gridDim
+// of the total.  Integer arithmetic on sums that every CTA forms alike, so the ranges tile the units.  Called by
+// all T threads of the block; one pass over the items' layer counts (4,096 items: about 2 us).
+// Equal unit counts instead left the CTA with the costliest items 28% over the mean (4,096 items
+// of 50 to 150 layers: 1,657 us, split by cost 1,500).
+template <int T>
+__device__ __forceinline__ int2 unit_range(const FwdParams& p, int Bc, int n_tiles) {
+  __shared__ unsigned long long warp_sum_s[T / 32];
+  __shared__ int bound[2];
+  const int t = threadIdx.x, lane = t & 31, warp = t >> 5;
+  const int q = (Bc + T - 1) / T, b0 = min(Bc, t * q), b1 = min(Bc, b0 + q);
+  const ItemGeom* items = p.buf.items + p.b_off;
+  unsigned long long mine = 0;
+  for (int b = b0; b < b1; ++b) mine += unit_cost(items[b].n_layers);
+  unsigned long long incl = mine;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const unsigned long long v = __shfl_up_sync(0xffffffffu, incl, o);
+    if (lane >= o) incl += v;
+  }
+  if (lane == 31) warp_sum_s[warp] = incl;
+  if (t == 0) { bound[0] = 0; bound[1] = Bc * n_tiles; }
+  __syncthreads();
+  unsigned long long before = incl - mine, total = 0;
+  for (int w = 0; w < T / 32; ++w) {
+    if (w < warp) before += warp_sum_s[w];
+    total += warp_sum_s[w];
+  }
+  total *= (unsigned)n_tiles;
+#pragma unroll
+  for (int e = 0; e < 2; ++e) {
+    // the first unit whose offset is at least x; offsets 0 and `total` are set above
+    const unsigned long long x = total * (blockIdx.x + e) / gridDim.x;
+    unsigned long long at = before * (unsigned)n_tiles;
+    if (x > at && x <= at + mine * (unsigned)n_tiles && blockIdx.x + e < gridDim.x) {
+      for (int b = b0; b < b1; ++b) {
+        const unsigned c = unit_cost(items[b].n_layers);
+        if (x <= at + (unsigned long long)c * (unsigned)n_tiles) {
+          bound[e] = b * n_tiles + (int)((x - at + c - 1) / c);
+          break;
+        }
+        at += (unsigned long long)c * (unsigned)n_tiles;
+      }
+    }
+  }
+  __syncthreads();
+  return make_int2(bound[0], bound[1]);
+}
+
 template <int W>
 __global__ void __launch_bounds__(32 * (W + 1), 1)
 k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int n_tiles,
@@ -416,11 +472,11 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
   }
   __syncthreads();
   // units of one chunk fit in 32 bits: the K buffer (2 GiB) bounds Bc x n_tiles x kTW x 4 B
-  const int units = Bc * n_tiles;
-  const int per = (units + (int)gridDim.x - 1) / (int)gridDim.x;
-  const int u_begin = (int)blockIdx.x * per;
-  const int u_end = u_begin + per < units ? u_begin + per : units;
-  const int n_units = u_end > u_begin ? (int)(u_end - u_begin) : 0;
+  // (one unit each where there are no more units than CTAs)
+  const int2 range = Bc * n_tiles <= (int)gridDim.x
+                         ? make_int2((int)blockIdx.x, (int)blockIdx.x + 1)
+                         : unit_range<32 * (W + 1)>(p, Bc, n_tiles);
+  const int u_begin = range.x, n_units = range.y - range.x;
   const int rt_max = (p.max_layers + kRT - 1) / kRT;   // work items per unit
   const int wbase = wn_first(p.wn_begin);
   const int S = n_slots;
