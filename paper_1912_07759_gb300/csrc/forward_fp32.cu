@@ -355,8 +355,11 @@ cudaError_t launch_opacity_p(const FwdParams& p, const CUtensorMap& sig, const C
 // equal cost, one per CTA (item-major, so consecutive units of a CTA mostly share the item and its
 // path lengths; a unit's cost grows with the square of its item's layer count).  A producer warp loads each unit's K tile [N][kTW] by 2-D TMA boxes of kCB rows
 // into one of up to three tile slots, plus the item's packed path lengths and annulus weights by
-// bulk copy when the item changes (after every earlier unit is done with them), on a barrier of
-// their own: a K tile of the item's second unit can land before them.  The W
+// bulk copy when the item changes, on a barrier of their own: a K tile of the item's second unit
+// can land before them.  Consecutive items' path lengths lie at the two ends of one area; where both
+// fit it, the next item's are loaded while the warps still work on this one, else once every unit of
+// this item is done (4,096 items of 50 to 150 layers, 945 wavenumbers: 1,500 us loaded always after
+// the item, K behind them; 1,467 so).  The W
 // contraction warps take work items (unit, 16-ray tile) from a shared counter, a unit's longest
 // tile first: tau = DL K for the tile's rays and its partial depth sum_j a_j (1 - e^-tau_j),
 // stored per tile.  The warp that completes a unit's last tile adds the tiles' partials in
@@ -365,16 +368,32 @@ cudaError_t launch_opacity_p(const FwdParams& p, const CUtensorMap& sig, const C
 // barrier over the CTA's warps: tiles of different lengths and units overlap freely.
 constexpr int kCB = 8;                           // K rows per TMA box
 constexpr int kMaxSlots = 3;                     // K-tile slots (units in flight per CTA)
+constexpr uint32_t kContractSmem = 226u * 1024u; // dynamic, beside under 1 KB of static
 
 struct ContractLayout {                          // dynamic shared memory (128-byte aligned)
-  uint32_t ktb, slot, dl, aj, total;             // slot i: K tile at i*slot, partials at +ktb
-  __host__ __device__ ContractLayout(int max_layers, int n_slots) {
+  uint32_t ktb, slot, dl, dl_area, aj, aj_bytes, total;   // slot i: K tile at i*slot, partials at +ktb
+  // limit: the bytes that the area of the path lengths may grow into (as far as two items need)
+  __host__ __device__ ContractLayout(int max_layers, int n_slots, uint32_t limit = 0) {
     ktb = (uint32_t)pad8(max_layers) * kTW * 4;
     const uint32_t ptb = (uint32_t)((max_layers + kRT - 1) / kRT) * kTW * 4;
     slot = ktb + ptb;
-    dl = (uint32_t)n_slots * slot;
-    aj = dl + (((uint32_t)dlp_offset(max_layers) * 4 + 127u) & ~127u);
-    total = aj + (((uint32_t)pad8(max_layers) * 4 + 127u) & ~127u) + 128u;
+    aj = (uint32_t)n_slots * slot;
+    aj_bytes = ((uint32_t)pad8(max_layers) * 4 + 127u) & ~127u;      // of each of two items
+    dl = aj + 2 * aj_bytes;
+    const uint32_t one = item_bytes(max_layers);
+    dl_area = one;
+    total = dl + dl_area + 128u;
+    if (limit > total) {
+      const uint32_t room = (limit - total) & ~127u;
+      const uint32_t more = room < one ? room : one;
+      dl_area += more;
+      total += more;
+    }
+  }
+  // the path lengths of an item of N layers, and where the item'th of a CTA keeps them
+  __host__ __device__ static uint32_t item_bytes(int N) { return ((uint32_t)dlp_offset(N) * 4 + 127u) & ~127u; }
+  __host__ __device__ uint32_t dl_at(int item, int N) const {
+    return dl + (item & 1 ? dl_area - item_bytes(N) : 0u);
   }
 };
 
@@ -451,21 +470,20 @@ __global__ void __launch_bounds__(32 * (W + 1), 1)
 k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int n_tiles,
                 int n_slots) {
   extern __shared__ unsigned char csm_raw[];
-  __shared__ __align__(8) uint64_t kfull[kMaxSlots], kempty[kMaxSlots], dlfull;
+  __shared__ __align__(8) uint64_t kfull[kMaxSlots], kempty[kMaxSlots], dlfull[2];
   __shared__ int abort_flag, next_item, done[kMaxSlots], slot_unit[kMaxSlots];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
-  const ContractLayout lay(p.max_layers, n_slots);
+  const ContractLayout lay(p.max_layers, n_slots, kContractSmem);
   unsigned char* base = reinterpret_cast<unsigned char*>(
       (reinterpret_cast<uintptr_t>(csm_raw) + 127) & ~(uintptr_t)127);
-  float* const DLP = reinterpret_cast<float*>(base + lay.dl);
-  float* const a_s = reinterpret_cast<float*>(base + lay.aj);
   if (threadIdx.x == 0) {
     for (int i = 0; i < kMaxSlots; ++i) {
       mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 1);
       done[i] = 0;
       slot_unit[i] = i;                                 // units 0 .. S-1 go to slots 0 .. S-1
     }
-    mbar_init(&dlfull, 1);
+    mbar_init(&dlfull[0], 1);
+    mbar_init(&dlfull[1], 1);
     abort_flag = 0;
     next_item = 0;
     mbar_fence_init();
@@ -484,8 +502,10 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
   if (warp == W) {
     // ---------------- producer
     if (lane != 0) return;
-    int dl_item = -1, dl_phases = 0;                    // dlfull: one phase per item
-    int k = 0;
+    // items of this CTA so far (dlfull[i & 1]: phase i / 2) and the last one's path-length bytes
+    int n_dl = 0;
+    uint32_t last_bytes = 0;
+    int k = 0, issued = 0;
     for (; k < n_units; ++k) {
       const int u = u_begin + k;
       const int bc = u / n_tiles, tile = u - bc * n_tiles;
@@ -493,37 +513,48 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
       const int N = p.buf.items[b].n_layers;
       const int sl = k % S, q = k / S;
       bool ok = q == 0 || mbar_wait_bounded(&kempty[sl], (q - 1) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
-      const bool new_item = b != dl_item;
-      // the units in the other slots must be done with the path lengths too
-      for (int d = 1; ok && new_item && d < S && d <= k; ++d) {
+      if (!ok || *(volatile int*)&abort_flag) { atomicExch(&abort_flag, 1); break; }
+      if (N == 0) {
+        mbar_arrive(&kfull[sl]);                           // nothing to load
+      } else {
+        const int nbox = (N + kCB - 1) / kCB;
+        mbar_arrive_expect_tx(&kfull[sl], (uint32_t)nbox * kCB * kTW * 4);
+        float* Kt = reinterpret_cast<float*>(base + sl * lay.slot);
+        for (int i = 0; i < nbox; ++i)
+          tma_load_2d(Kt + (size_t)i * kCB * kTW, &tm_k, 0, (bc * n_tiles + tile) * p.max_layers + i * kCB,
+                      &kfull[sl]);
+      }
+      issued = k + 1;
+      const int item = bc - u_begin / n_tiles;             // of this CTA
+      if (item < n_dl) continue;
+      // the units in the other slots that still read where this item's path lengths go must be
+      // done: those of the item before the last, and of the last where the two do not fit
+      const uint32_t bytes = ContractLayout::item_bytes(N);
+      const bool beside = last_bytes + bytes <= lay.dl_area;
+      for (int d = 1; ok && d < S && d <= k; ++d) {
         const int kp = k - d;
-        ok = mbar_wait_bounded(&kempty[kp % S], (kp / S) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
+        if (!beside || (u_begin + kp) / n_tiles - u_begin / n_tiles < item - 1)
+          ok = mbar_wait_bounded(&kempty[kp % S], (kp / S) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
       }
       if (!ok || *(volatile int*)&abort_flag) { atomicExch(&abort_flag, 1); break; }
-      if (new_item) {
-        dl_item = b;
-        ++dl_phases;
-        if (N == 0) {
-          mbar_arrive(&dlfull);
-        } else {
-          mbar_arrive_expect_tx(&dlfull, (uint32_t)(dlp_offset(N) * 4 + p.buf.npad * 4));
-          bulk_g2s(DLP, p.buf.dlp + (size_t)b * dlp_offset(p.max_layers),
-                   (uint32_t)(dlp_offset(N) * 4), &dlfull);
-          bulk_g2s(a_s, p.buf.aj + (size_t)b * p.buf.npad, (uint32_t)(p.buf.npad * 4), &dlfull);
-        }
+      uint64_t* full = &dlfull[item & 1];
+      if (N == 0) {
+        mbar_arrive(full);
+      } else {
+        mbar_arrive_expect_tx(full, (uint32_t)(dlp_offset(N) * 4 + p.buf.npad * 4));
+        bulk_g2s(base + lay.dl_at(item, N), p.buf.dlp + (size_t)b * dlp_offset(p.max_layers),
+                 (uint32_t)(dlp_offset(N) * 4), full);
+        bulk_g2s(base + lay.aj + (item & 1) * lay.aj_bytes, p.buf.aj + (size_t)b * p.buf.npad,
+                 (uint32_t)(p.buf.npad * 4), full);
       }
-      if (N == 0) { mbar_arrive(&kfull[sl]); continue; }   // nothing to load
-      const int nbox = (N + kCB - 1) / kCB;
-      mbar_arrive_expect_tx(&kfull[sl], (uint32_t)nbox * kCB * kTW * 4);
-      float* Kt = reinterpret_cast<float*>(base + sl * lay.slot);
-      for (int i = 0; i < nbox; ++i)
-        tma_load_2d(Kt + (size_t)i * kCB * kTW, &tm_k, 0, (bc * n_tiles + tile) * p.max_layers + i * kCB,
-                    &kfull[sl]);
+      n_dl = item + 1;
+      last_bytes = bytes;
     }
     // every copy issued has landed before the CTA may exit
-    if (dl_phases > 0) mbar_wait_bounded(&dlfull, (dl_phases - 1) & 1, nullptr, 0);
-    for (int i = 0; i < S && i < k; ++i) {
-      const int kl = k - 1 - i;
+    for (int i = 0; i < 2 && i < n_dl; ++i)
+      mbar_wait_bounded(&dlfull[(n_dl - 1 - i) & 1], ((n_dl - 1 - i) >> 1) & 1, nullptr, 0);
+    for (int i = 0; i < S && i < issued; ++i) {
+      const int kl = issued - 1 - i;
       mbar_wait_bounded(&kfull[kl % S], (kl / S) & 1, nullptr, 0);
     }
     return;
@@ -548,19 +579,22 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
     const int sl = k % S, q = k / S;
     // the slot holds unit k - S until that unit's last tile hands it over; only then is
     // phase q the one kfull[sl] is in (a warp may take work of later units early)
-    // then the item's path lengths: dlfull's phase is the item's ordinal in this CTA, and the
-    // next item's starts only when every unit of this one is done
+    // then the item's path lengths: the phase of its dlfull counts every second item of this CTA,
+    // and the next one's starts only when every unit of this item is done
+    const int item = bc - u_begin / n_tiles;
     const bool ok = __all_sync(0xffffffffu, wait_slot(&slot_unit[sl], k, &abort_flag, p.dev_err) &&
                                                 mbar_wait_bounded(&kfull[sl], q & 1, p.dev_err,
                                                                   TR_DEVERR_TIMEOUT) &&
-                                                mbar_wait_bounded(&dlfull, (bc - u_begin / n_tiles) & 1,
+                                                mbar_wait_bounded(&dlfull[item & 1], (item >> 1) & 1,
                                                                   p.dev_err, TR_DEVERR_TIMEOUT) &&
                                                 !*(volatile int*)&abort_flag);
     if (!ok) { if (lane == 0) atomicExch(&abort_flag, 1); return; }
     float* part = reinterpret_cast<float*>(base + sl * lay.slot + lay.ktb);
     if (N > 0) {
       float pt[4];
-      contract_tile(N, t * kRT, reinterpret_cast<const float*>(base + sl * lay.slot), DLP, a_s, pt);
+      contract_tile(N, t * kRT, reinterpret_cast<const float*>(base + sl * lay.slot),
+                    reinterpret_cast<const float*>(base + lay.dl_at(item, N)),
+                    reinterpret_cast<const float*>(base + lay.aj + (item & 1) * lay.aj_bytes), pt);
       *reinterpret_cast<float4*>(part + t * kTW + 4 * lane) = make_float4(pt[0], pt[1], pt[2], pt[3]);
     }
     __syncwarp();
@@ -687,12 +721,11 @@ cudaError_t launch_contract_fp32(const FwdParams& p, int Bc, const float* kbuf, 
   if (!encode_2d_f32(&tm, kbuf, kTW, (unsigned long long)Bc * tiles * p.max_layers, kTW * 4, kTW,
                      kCB))
     return cudaErrorInvalidValue;
-  constexpr uint32_t kSmemMax = 227u * 1024u;
   // as many K-tile slots as fit, up to three (the next units' loads overlap the contraction)
   int slots = kMaxSlots;
-  while (slots > 1 && ContractLayout(p.max_layers, slots).total > kSmemMax) --slots;
-  const uint32_t smem = ContractLayout(p.max_layers, slots).total;
-  if (smem > kSmemMax) return cudaErrorInvalidConfiguration;
+  while (slots > 1 && ContractLayout(p.max_layers, slots).total > kContractSmem) --slots;
+  const uint32_t smem = ContractLayout(p.max_layers, slots, kContractSmem).total;
+  if (smem > kContractSmem) return cudaErrorInvalidConfiguration;
   // eleven contraction warps (twelve plus the producer would be held to 128 registers and
   // spill; eleven keep 168), or eight
   if (kind == kContractFfma11) return launch_contract_t<11>(p, tm, Bc, tiles, slots, smem, s);
