@@ -802,6 +802,71 @@ __global__ void k_adjoint_sum(TileSumArgs ts, int B) {
   }
 }
 
+// Sums of the wavenumber tiles' partial sums into the row's first slot, in tile
+// order and compensated as below, four consecutive elements a thread (of G_DL the groups that reach
+// the diagonal or lie above it, which alone are read afterwards), 16 bytes a tile, no division by
+// the array sizes.  For launches of several waves of such threads: 15 tiles of 1,024 items 123 us
+// (135 by the kernel below), the few tiles of each of 50 Jacobian rows of 128 items 88 us (221).
+// With fewer items the threads are too few: 58 tiles of 8 items 21 us (10), 296 tiles of two runs
+// of 160 items 798 us (639).
+struct TileSum4Args {
+  float *dl, *a, *f, *rp;
+  int npad, n_f, slots;           // slots per item
+  RowGroup rows;                  // n_rows == 0: one row of all slots
+};
+constexpr int kSumThreads = 256;
+constexpr long long kSum4Threads = 1 << 20;            // about four waves of the GPU's threads
+__device__ __forceinline__ float kahan(float s, float& c, float v) {
+  const float y = __fsub_rn(v, c);
+  const float u = __fadd_rn(s, y);
+  c = __fsub_rn(__fsub_rn(u, s), y);
+  return u;
+}
+__device__ __forceinline__ void sum_tiles4(float* p, size_t stride, int tiles) {
+  float4 s = *reinterpret_cast<const float4*>(p), c = make_float4(0.f, 0.f, 0.f, 0.f);
+#pragma unroll 4
+  for (int t = 1; t < tiles; ++t) {
+    const float4 v = *reinterpret_cast<const float4*>(p + t * stride);
+    s.x = kahan(s.x, c.x, v.x); s.y = kahan(s.y, c.y, v.y);
+    s.z = kahan(s.z, c.z, v.z); s.w = kahan(s.w, c.w, v.w);
+  }
+  *reinterpret_cast<float4*>(p) = s;
+}
+__device__ __forceinline__ void sum_tiles1(float* p, size_t stride, int tiles) {
+  float s = *p, c = 0.f;
+#pragma unroll 4
+  for (int t = 1; t < tiles; ++t) s = kahan(s, c, p[t * stride]);
+  *p = s;
+}
+__host__ __device__ inline int sum_units(int npad, int n_f) {
+  return npad * npad / 4 + npad / 4 + (n_f % 4 == 0 ? n_f / 4 : n_f) + 1;
+}
+__global__ void __launch_bounds__(kSumThreads) k_adjoint_sum4(TileSum4Args ts) {
+  const int b = blockIdx.y, r = blockIdx.z, npad = ts.npad;
+  const int s0 = ts.rows.n_rows > 0 ? ts.rows.slot0[r] : 0;
+  const int tiles = (ts.rows.n_rows > 0 ? ts.rows.slot0[r + 1] : ts.slots) - s0;
+  if (tiles < 2) return;
+  const size_t slot = (size_t)b * ts.slots + s0;
+  const int q = npad / 4;                               // groups of a G_DL row
+  int u = blockIdx.x * kSumThreads + threadIdx.x;
+  if (u < npad * q) {
+    const int j = u / q, l = 4 * (u - j * q);
+    const size_t m = (size_t)npad * npad;
+    if (l + 3 >= j) sum_tiles4(ts.dl + slot * m + 4 * (size_t)u, m, tiles);
+    return;
+  }
+  u -= npad * q;
+  if (u < q) return sum_tiles4(ts.a + slot * npad + 4 * u, npad, tiles);
+  u -= q;
+  const bool by4 = ts.n_f % 4 == 0;                     // else a slot's features are not 16-byte aligned
+  const int n_f = by4 ? ts.n_f / 4 : ts.n_f;
+  if (u < n_f) {
+    float* f = ts.f + slot * ts.n_f;
+    return by4 ? sum_tiles4(f + 4 * u, ts.n_f, tiles) : sum_tiles1(f + u, ts.n_f, tiles);
+  }
+  if (u == n_f) sum_tiles1(ts.rp + slot, 1, tiles);
+}
+
 struct ItemParams {
   GeomParams gp;
   const double* theta; int n_theta;
@@ -1281,15 +1346,23 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
       // the tiles' partial sums into the rows' first slots by a GPU-wide pass, so the
       // per-atmosphere kernel reads one set of sums
       KernelTimer kt(ctx, "k_adjoint_sum", s);
-      TileSumArgs ts{};
-      ts.arr[0] = part_a;  ts.m[0] = npad;
-      ts.arr[1] = part_dl; ts.m[1] = (long long)npad * npad; ts.tri[1] = npad;
-      ts.arr[2] = part_f;  ts.m[2] = (long long)d->max_layers * n_feat;
-      ts.arr[3] = part_rp; ts.m[3] = 1;
-      ts.slots = slots; ts.rows = rows;
-      const long long most = (long long)bc * npad * npad;
-      const int gx = (int)std::max<long long>(1, std::min<long long>((most + 255) / 256, 8LL * n_sm));
-      k_adjoint_sum<<<dim3(gx, 4, n_rows), 256, 0, s>>>(ts, bc);
+      const int n_f = d->max_layers * n_feat, units = sum_units(npad, n_f);
+      if ((long long)bc * n_rows * units >= kSum4Threads) {
+        TileSum4Args ts{};
+        ts.dl = part_dl; ts.a = part_a; ts.f = part_f; ts.rp = part_rp;
+        ts.npad = npad; ts.n_f = n_f; ts.slots = slots; ts.rows = rows;
+        k_adjoint_sum4<<<dim3((units + kSumThreads - 1) / kSumThreads, bc, n_rows), kSumThreads, 0, s>>>(ts);
+      } else {
+        TileSumArgs ts{};
+        ts.arr[0] = part_a;  ts.m[0] = npad;
+        ts.arr[1] = part_dl; ts.m[1] = (long long)npad * npad; ts.tri[1] = npad;
+        ts.arr[2] = part_f;  ts.m[2] = (long long)d->max_layers * n_feat;
+        ts.arr[3] = part_rp; ts.m[3] = 1;
+        ts.slots = slots; ts.rows = rows;
+        const long long most = (long long)bc * npad * npad;
+        const int gx = (int)std::max<long long>(1, std::min<long long>((most + 255) / 256, 8LL * n_sm));
+        k_adjoint_sum<<<dim3(gx, 4, n_rows), 256, 0, s>>>(ts, bc);
+      }
       err = cudaGetLastError();
       if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint sum kernel: ") + cudaGetErrorString(err));
     }

@@ -3,9 +3,9 @@
 //
 // tr_capture_forward_batch
 //   1. autotune (optional): every configuration of the forward's search space (ForwardChoice:
-//      the two-stage form with 3, 2 or 1 opacity CTAs per SM and the ring depth that leaves,
-//      times (FP32) the contraction as one CTA per SM with two K tiles or two CTAs per SM with
-//      one, or the fused FP32 kernel) is run on the caller's own inputs -- one untimed run, then
+//      the two-stage form with as many opacity CTAs per SM as fit, 2 or 1, and the ring depth
+//      that leaves, times (FP32, more than 112 layers) the FFMA contraction with 8 or 11 warps,
+//      or the fused FP32 kernel) is run on the caller's own inputs -- one untimed run, then
 //      kTuneReps runs timed with CUDA events on the caller's stream -- and the fastest median
 //      wins; it is remembered on the context for this batch shape, so plain
 //      tr_forward_transit_batch calls of the same shape use it too;

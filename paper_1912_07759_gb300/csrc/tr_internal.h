@@ -387,7 +387,7 @@ int set_error(tr_ctx* ctx, int code, const std::string& msg);
 // kernels (the default when kbuf is given; also used when the fused kernel's shared memory
 // does not fit) or the fused kernel (without kbuf, or when `choice` asks for it); mixed
 // precision always takes the two-stage form (tensor-core contraction).  per_sm: CTAs per SM of
-// the two-stage opacity kernel (0 = as many as fit, up to 3); stages: ring depth cap of the
+// the two-stage opacity kernel (0 = as many as fit, up to 6; 3 with the exponential scheme); stages: ring depth cap of the
 // fused kernel (0 = the deepest that fits); contract_per_sm: the FP32 two-stage contraction
 // (launch_contract_fp32's kind).
 enum { kFormTwoStage = 0, kFormFused = 1 };

@@ -46,3 +46,28 @@ def test_gradient_at_tile_edges(n_mol, with_cia, with_ray, most, layers):
         g, ref = grad[b].cpu().numpy(), gbin[b] @ jac
         floor = 1e-3 * np.abs(ref).max()
         assert (np.abs(g - ref) <= 1e-4 * np.maximum(np.abs(ref), floor)).all(), (n, g, ref)
+
+
+def test_tile_sums_of_a_large_batch_equal_a_small_one():
+    """The tile sums of launches large enough take four elements a thread, features one at a time
+    where a slot's are not a multiple of four (33 layers of 9): the same sums, bit for bit."""
+    import torch
+    from paper_1912_07759_gb300 import transit as T
+    ctx = T.TransitContext(0)
+    tb = S.make_tables(5, 2, 4, 5, 3000, with_cia=False)
+    tables = T.XsecTables(ctx, tb)
+    bins_h = S.bins_logspaced(6)
+    bins = T.Bins(ctx, tables, *bins_h)
+    spec_h = S.batch_spec(2)
+    B = 1500
+    spec = T.BatchSpec(spec_h, max_layers=33)
+    th = torch.tensor(S.draw_theta(41, B, spec_h), device="cuda")
+    nl = torch.tensor(np.random.default_rng(1).integers(1, 34, B).astype(np.int32), device="cuda")
+    gbin = torch.tensor(np.random.default_rng(2).normal(size=(B, 6)), device="cuda")
+    _, grad, _, _ = T.adjoint_transit(ctx, tables, spec, th, nl, bins, gbin=gbin, want_binned=False)
+    for b in (0, 700, 1488):
+        part = slice(b, b + 12)
+        _, g, _, _ = T.adjoint_transit(ctx, tables, spec, th[part].contiguous(), nl[part].contiguous(),
+                                       bins, gbin=gbin[part].contiguous(), want_binned=False)
+        assert torch.equal(g, grad[part]), b
+    ctx.sync_status()
