@@ -100,6 +100,7 @@ __device__ __forceinline__ float tf32_hi(float x) {
 // of the geometry kernel's layer-major DL.
 __global__ void __launch_bounds__(128)
 k_dl_tf32(ItemBuffers buf, int max_layers, int n_cm, float* __restrict__ tiles) {
+  pdl_wait();                                               // the path lengths are written
   const int b = blockIdx.y;
   const int q = 4 * blockIdx.x + (threadIdx.x >> 5);        // core matrix of this warp
   if (q >= n_cm) return;
@@ -112,7 +113,7 @@ k_dl_tf32(ItemBuffers buf, int max_layers, int n_cm, float* __restrict__ tiles) 
   const int j = 8 * (rem >> 1) + r, l = 8 * (2 * m + odd) + 4 * (rem & 1) + c;
   const int N = buf.items[b].n_layers;
   const float* dlt = buf.dlt + (size_t)b * max_layers * buf.npad;
-  const float x = (l < N && j <= l) ? __ldg(dlt + (size_t)l * buf.npad + j) : 0.f;
+  const float x = (l < N && j <= l) ? dlt[(size_t)l * buf.npad + j] : 0.f;
   const float h = tf32_hi(x);
   float* hi = tiles + ((size_t)b * 2 * n_cm + q) * 32;
   hi[lane] = h;                                             // row r, column c: 4 r + c = lane
@@ -379,6 +380,9 @@ cudaError_t launch_dl_tf32(const ItemBuffers& buf, int B, int max_layers, void* 
   if (B <= 0) return cudaSuccess;
   if (!tc_contract_fits(max_layers)) return cudaErrorInvalidValue;
   const int n_cm = dl_cores(pad16i(max_layers) / 8);
+  if (B < kFewAtmospheres)                                  // as k_pathlen before it
+    return launch_dependent(k_dl_tf32, dim3((n_cm + 3) / 4, B), dim3(128), 0, s, buf, max_layers,
+                            n_cm, static_cast<float*>(tiles));
   k_dl_tf32<<<dim3((n_cm + 3) / 4, B), 128, 0, s>>>(buf, max_layers, n_cm,
                                                     static_cast<float*>(tiles));
   return cudaGetLastError();

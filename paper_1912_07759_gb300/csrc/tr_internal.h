@@ -131,6 +131,8 @@ struct ItemBuffers {
 
 __host__ __device__ inline int pad8(int n) { return (n + 7) & ~7; }
 
+constexpr int kFewAtmospheres = 16;      // fewer: the short geometry kernels are launch-bound
+
 // Programmatic dependent launch.  A kernel launched by launch_dependent may start while the
 // kernel before it in the stream is still running (once every CTA of that kernel has called
 // pdl_trigger, or exited); it must call pdl_wait before it reads anything earlier work wrote
