@@ -470,7 +470,7 @@ __global__ void __launch_bounds__(32 * (W + 1), 1)
 k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, int n_tiles,
                 int n_slots) {
   extern __shared__ unsigned char csm_raw[];
-  __shared__ __align__(8) uint64_t kfull[kMaxSlots], kempty[kMaxSlots], dlfull[2];
+  __shared__ __align__(8) uint64_t kfull[kMaxSlots], kempty[kMaxSlots], dlfull[kMaxSlots];
   __shared__ int abort_flag, next_item, done[kMaxSlots], slot_unit[kMaxSlots];
   const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
   const ContractLayout lay(p.max_layers, n_slots, kContractSmem);
@@ -478,12 +478,10 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
       (reinterpret_cast<uintptr_t>(csm_raw) + 127) & ~(uintptr_t)127);
   if (threadIdx.x == 0) {
     for (int i = 0; i < kMaxSlots; ++i) {
-      mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 1);
+      mbar_init(&kfull[i], 1); mbar_init(&kempty[i], 1); mbar_init(&dlfull[i], 1);
       done[i] = 0;
       slot_unit[i] = i;                                 // units 0 .. S-1 go to slots 0 .. S-1
     }
-    mbar_init(&dlfull[0], 1);
-    mbar_init(&dlfull[1], 1);
     abort_flag = 0;
     next_item = 0;
     mbar_fence_init();
@@ -502,7 +500,8 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
   if (warp == W) {
     // ---------------- producer
     if (lane != 0) return;
-    // items of this CTA so far (dlfull[i & 1]: phase i / 2) and the last one's path-length bytes
+    // items of this CTA so far (item i: phase i / kMaxSlots of dlfull[i % kMaxSlots]) and the last
+    // one's path-length bytes
     int n_dl = 0;
     uint32_t last_bytes = 0;
     int k = 0, issued = 0;
@@ -537,7 +536,7 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
           ok = mbar_wait_bounded(&kempty[kp % S], (kp / S) & 1, p.dev_err, TR_DEVERR_TIMEOUT);
       }
       if (!ok || *(volatile int*)&abort_flag) { atomicExch(&abort_flag, 1); break; }
-      uint64_t* full = &dlfull[item & 1];
+      uint64_t* full = &dlfull[item % kMaxSlots];
       if (N == 0) {
         mbar_arrive(full);
       } else {
@@ -551,8 +550,10 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
       last_bytes = bytes;
     }
     // every copy issued has landed before the CTA may exit
-    for (int i = 0; i < 2 && i < n_dl; ++i)
-      mbar_wait_bounded(&dlfull[(n_dl - 1 - i) & 1], ((n_dl - 1 - i) >> 1) & 1, nullptr, 0);
+    for (int i = 0; i < kMaxSlots && i < n_dl; ++i) {
+      const int il = n_dl - 1 - i;
+      mbar_wait_bounded(&dlfull[il % kMaxSlots], (il / kMaxSlots) & 1, nullptr, 0);
+    }
     for (int i = 0; i < S && i < issued; ++i) {
       const int kl = issued - 1 - i;
       mbar_wait_bounded(&kfull[kl % S], (kl / S) & 1, nullptr, 0);
@@ -578,15 +579,20 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
     if (t >= target) continue;                          // beyond this item's rays
     const int sl = k % S, q = k / S;
     // the slot holds unit k - S until that unit's last tile hands it over; only then is
-    // phase q the one kfull[sl] is in (a warp may take work of later units early)
-    // then the item's path lengths: the phase of its dlfull counts every second item of this CTA,
-    // and the next one's starts only when every unit of this item is done
+    // phase q the one kfull[sl] is in (a warp may take work of later units early);
+    // then the item's path lengths.  A parity wait tells a phase from the one before it only once
+    // the phase before that is over: here item - kMaxSlots's, whose first unit is at most
+    // k - kMaxSlots.  K of unit k has landed, so the producer has seen every unit up to k - S done,
+    // that one among them.  (Two barriers are too few: with one unit per item and S = 3, three items
+    // are in flight, and a wait for the third returns at once while the first one's path lengths are
+    // still arriving.)  The next phase starts only when every unit of this item is done
     const int item = bc - u_begin / n_tiles;
     const bool ok = __all_sync(0xffffffffu, wait_slot(&slot_unit[sl], k, &abort_flag, p.dev_err) &&
                                                 mbar_wait_bounded(&kfull[sl], q & 1, p.dev_err,
                                                                   TR_DEVERR_TIMEOUT) &&
-                                                mbar_wait_bounded(&dlfull[item & 1], (item >> 1) & 1,
-                                                                  p.dev_err, TR_DEVERR_TIMEOUT) &&
+                                                mbar_wait_bounded(&dlfull[item % kMaxSlots],
+                                                                  (item / kMaxSlots) & 1, p.dev_err,
+                                                                  TR_DEVERR_TIMEOUT) &&
                                                 !*(volatile int*)&abort_flag);
     if (!ok) { if (lane == 0) atomicExch(&abort_flag, 1); return; }
     float* part = reinterpret_cast<float*>(base + sl * lay.slot + lay.ktb);
