@@ -27,6 +27,7 @@
 #include <cuda_fp16.h>
 #include <type_traits>
 #include "tma.h"
+#include "sum3.h"
 #include "tr_internal.h"
 
 namespace tr {
@@ -904,24 +905,17 @@ struct ItemSmem {
   }
 };
 
-// Adds t to the double-float sum (hi, lo): Knuth's TwoSum, the remainders collected in lo.
-__device__ __forceinline__ void add_df(float& hi, float& lo, float t) {
-  const float s = __fadd_rn(hi, t);
-  const float bb = __fsub_rn(s, hi);
-  lo = __fadd_rn(lo, __fadd_rn(__fsub_rn(hi, __fsub_rn(s, bb)), __fsub_rn(t, bb)));
-  hi = s;
-}
-
 // One CTA per (atmosphere, row).  GB300 runs FP64 at a small fraction of its FP32 rate and with
 // long latency (the SM completes one FP64 warp instruction per 19 cycles, a dependent one takes
 // about 140), so the kernel is bound by its FP64 instructions in large batches and by their
 // chains in small ones.  Four warps take the layers' terms in FP64 while the other four take the
 // O(N^2) path-length sensitivities, FP32 terms (from double-float altitudes, as the forward path
-// lengths) added into double-float sums without an FP64 instruction; the backward hydrostatic
+// lengths) added to FP64 accuracy without an FP64 instruction (sum3.h); the backward hydrostatic
 // recursion is a scan of its linear steps, and a warp adds each of the CTA's sums.  The G_DL
 // matrix and the features are staged in shared memory by coalesced reads (gathered from L2 by one
 // thread per radius they held the kernel at 112 us whatever the batch).  100 layers, 5 absorbers:
-// 8 atmospheres 114 -> 37 us, 1,024 193 -> 140 us, 50 rows of 128 atmospheres 5.58 -> 0.70 ms.
+// 8 atmospheres 114 -> 39 us, 1,024 193 -> 144 us, 50 rows of 128 atmospheres 5.58 -> 0.75 ms (of
+// which the third part of the sums, without which they keep 48 bits, 2, 7 and 45 us).
 __global__ void __launch_bounds__(kItemThreads)
 k_adjoint_item(ItemParams ip) {
   extern __shared__ double dsm[];
@@ -999,7 +993,7 @@ k_adjoint_item(ItemParams ip) {
   // ---- radii from path lengths and annulus weights
   //      DL[j][l] = 2 (s(l+1,j) - s(l,j)), s(k,j) = sqrt(r_k^2 - r_j^2):
   //      ds(k,j)/dr_k = r_k / s,  ds(k,j)/dr_j = -r_j / s;  r_k^2 - r_j^2 = (z_k - z_j)(r_k + r_j)
-  //      with z_k - z_j from the double-float altitudes; each term in FP32, sums in double-float
+  //      with z_k - z_j from the double-float altitudes; each term in FP32, sums to FP64
   const double dln = (gp.ln_pmin - gp.ln_pmax) / N;
   const int f_dS = nm, f_R = 2 * nm, f_C = 2 * nm + ns, f_dC = f_C + nq, f_K = f_dC + nq;
   double acc[TR_MAX_SPECIES + 3];                   // species, cloud top, d/dcz, d/dR_p
@@ -1009,27 +1003,31 @@ k_adjoint_item(ItemParams ip) {
     for (int k = t - kItemHalf; k <= N; k += kItemHalf) {
       const float2 zk = zs[k];
       const float rk = rs[k];
-      float hi = 0.f, lo = 0.f;
-      float below = 0.f;                            // G[j][k]
-      for (int j = 0; j < k; ++j) {                 // k as the outer radius of s(k, j)
-        below = k < N ? G[j * pitch + k] : 0.f;
-        const float gs = 2.f * (G[j * pitch + k - 1] - below);
-        const float2 zj = zs[j];
-        const float s2 = diff_df(zk.x, zk.y, zj.x, zj.y) * (rk + rs[j]);
-        add_df(hi, lo, gs != 0.f ? gs * rk * rsqrtf(s2) : 0.f);
-      }
-      float left = k < N ? G[k * pitch + k] : 0.f;  // G[k][kk - 1]
-      for (int kk = k + 1; kk <= N; ++kk) {         // k as the ray of s(kk, k)
-        const float right = kk < N ? G[k * pitch + kk] : 0.f;
-        const float gs = 2.f * (left - right);
-        left = right;
-        const float2 zu = zs[kk];
-        const float s2 = diff_df(zu.x, zu.y, zk.x, zk.y) * (rs[kk] + rk);
-        add_df(hi, lo, gs != 0.f ? -(gs * rk * rsqrtf(s2)) : 0.f);
-      }
+      const double paths = sum_fp32_terms([&](auto add) {   // two terms at a time
+        auto outer = [&](int j) {                   // k as the outer radius of s(k, j), j < k
+          const float gs = 2.f * (G[j * pitch + k - 1] - (k < N ? G[j * pitch + k] : 0.f));
+          const float2 zj = zs[j];
+          const float s2 = diff_df(zk.x, zk.y, zj.x, zj.y) * (rk + rs[j]);
+          return gs != 0.f ? gs * rk * rsqrtf(s2) : 0.f;
+        };
+        for (int j = 0; j < k; j += 2) add(outer(j), j + 1 < k ? outer(j + 1) : 0.f);
+        auto ray = [&](int u, float dg) {           // k as the ray of s(u, k), u > k
+          const float gs = 2.f * dg;
+          const float2 zu = zs[u];
+          const float s2 = diff_df(zu.x, zu.y, zk.x, zk.y) * (rs[u] + rk);
+          return gs != 0.f ? -(gs * rk * rsqrtf(s2)) : 0.f;
+        };
+        float g0 = k < N ? G[k * pitch + k] : 0.f;  // G[k][u - 1]
+        for (int u = k + 1; u <= N; u += 2) {
+          const float g1 = u < N ? G[k * pitch + u] : 0.f, g2 = u + 1 < N ? G[k * pitch + u + 1] : 0.f;
+          const float t = ray(u, g0 - g1);
+          add(t, u < N ? ray(u + 1, g1 - g2) : 0.f);
+          g0 = g2;
+        }
+      });
       // a_j = (r_{j+1}^2 - r_j^2) / R_s^2
       const double ga = ((k >= 1 ? Ga[k - 1] : 0.0) - (k < N ? Ga[k] : 0.0));
-      Gr[k] = fma(ga * 2.0 * (rp + z[k]), inv_rs2, (double)hi + (double)lo);
+      Gr[k] = fma(ga * 2.0 * (rp + z[k]), inv_rs2, paths);
     }
   } else {
     // ---- per layer: opacity weights, densities, cloud; recursion factors; T-node weights
