@@ -22,6 +22,9 @@
  *  - `stream` is a cudaStream_t passed as void* (NULL = the legacy default stream).  Calls
  *    that take a stream are asynchronous on it and never synchronise the device, except
  *    where stated.  A context is not thread-safe; use one per host thread.
+ *  - Batch calls may be captured into a CUDA graph (with a workspace given).  Such a call holds
+ *    the context's second stream until its capture ends; calls on streams outside the capture
+ *    work meanwhile, without that stream.
  *  - There is no CPU fallback: without a usable CUDA device every call fails.
  */
 #ifndef TRANSIT_H_

@@ -1253,7 +1253,7 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   ItemBuffers buf; double* depth = nullptr; char* extra = nullptr;
   // the altitudes and path lengths on a second branch beside the first opacity kernel
   Fork fk;
-  Fork* fork = fork_ready(ctx, &fk) ? &fk : nullptr;
+  Fork* fork = fork_ready(ctx, &fk, s) ? &fk : nullptr;
   int rc = prepare_batch(ctx, t, d, n_in, need, B, d_theta, d_nlayers, d_status, ws, ws_bytes,
                          s, &buf, &depth, &extra, fork);
   if (rc != TR_OK) return rc;

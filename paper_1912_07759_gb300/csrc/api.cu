@@ -268,7 +268,7 @@ extern "C" void tr_destroy(tr_ctx* ctx) {
   delete ctx;
 }
 
-bool tr::fork_ready(tr_ctx* ctx, Fork* f) {
+bool tr::fork_ready(tr_ctx* ctx, Fork* f, cudaStream_t s) {
   if (!ctx->aux) {
     int least = 0, greatest = 0;
     cudaDeviceGetStreamPriorityRange(&least, &greatest);
@@ -284,6 +284,17 @@ bool tr::fork_ready(tr_ctx* ctx, Fork* f) {
       return false;
     }
     ctx->aux = st; ctx->ev_fork = a; ctx->ev_join = b;
+  }
+  // a capture that a call of this context takes part in holds the auxiliary stream until it ends:
+  // a call on a stream outside that capture does without the branch
+  cudaStreamCaptureStatus held = cudaStreamCaptureStatusNone, mine = cudaStreamCaptureStatusNone;
+  unsigned long long held_id = 0, mine_id = 0;
+  if (cudaStreamGetCaptureInfo(ctx->aux, &held, &held_id) != cudaSuccess ||
+      (held != cudaStreamCaptureStatusNone &&
+       (cudaStreamGetCaptureInfo(s, &mine, &mine_id) != cudaSuccess ||
+        held != cudaStreamCaptureStatusActive || mine != held || mine_id != held_id))) {
+    cudaGetLastError();
+    return false;
   }
   f->aux = ctx->aux;
   f->open = f->pending = false;
@@ -1136,7 +1147,7 @@ int tr::forward_batch_impl(tr_ctx* ctx, const tr_tables* t, const tr_batch_desc*
   ItemBuffers buf; double* depth = nullptr; char* extra = nullptr;
   // the path-length kernels on a second branch beside the opacity kernel
   Fork fk;
-  Fork* fork = fork_ready(ctx, &fk) ? &fk : nullptr;
+  Fork* fork = fork_ready(ctx, &fk, s) ? &fk : nullptr;
   int rc = prepare_batch(ctx, t, d, n_in, need, B, d_theta, d_nlayers, d_status, ws, ws_bytes,
                          s, &buf, &depth, &extra, fork);
   if (rc != TR_OK) { join_fork(ctx, fork, s); return rc; }

@@ -282,7 +282,7 @@ extern "C" int tr_forward_emission_batch(tr_ctx* ctx, const tr_tables* t,
   ItemBuffers buf; double* depth = nullptr; char* extra = nullptr;
   Fork fk;
   fk.pathlen = false;
-  Fork* fork = fork_ready(ctx, &fk) ? &fk : nullptr;
+  Fork* fork = fork_ready(ctx, &fk, s) ? &fk : nullptr;
   rc = prepare_batch(ctx, t, d, n_in, need, B, d_theta, d_nlayers, d_status, ws, ws_bytes, s,
                      &buf, &depth, &extra, fork);
   if (rc != TR_OK) return rc;

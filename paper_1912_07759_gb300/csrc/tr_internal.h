@@ -364,9 +364,10 @@ struct Fork {
   int B = 0;
   ItemBuffers buf{};
 };
-// Creates the auxiliary stream and its events on first use; false when that fails (the
-// forward then runs on the caller's stream alone).
-bool fork_ready(tr_ctx* ctx, Fork* f);
+// Creates the auxiliary stream and its events on first use.  False when that fails, or while the
+// auxiliary stream belongs to an open capture that stream s is not in: the call then runs on the
+// caller's stream alone.
+bool fork_ready(tr_ctx* ctx, Fork* f, cudaStream_t s);
 // Issues the pending path-length kernel: on the branch (detached) or on s.
 cudaError_t fork_start(tr_ctx* ctx, Fork* f, cudaStream_t s, bool detached);
 void join_fork(tr_ctx* ctx, Fork* f, cudaStream_t s);
