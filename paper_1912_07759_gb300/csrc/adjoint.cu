@@ -63,6 +63,7 @@ struct AdjParams {
   const double* inv_dtc;          // [n_t_cia - 1]
   const float* gd;                // [B][n_in] dL/dD at the native wavenumbers of the range
   int n_in, tiles, n_feat;        // tiles: slots per item of the partial sums
+  unsigned items;                 // of the launch
   unsigned ray_mask;              // species with Rayleigh cross-sections that are not all zero
   float* part_a;                  // [B][tiles][npad]
   float* part_dl;                 // [B][tiles][npad][npad]  (ray j, shell l), j <= l
@@ -220,7 +221,7 @@ struct AdjSmem {
   }
 };
 
-// One CTA per (item, 64-wavenumber tile); grid (items, tiles).  Bound by instruction latency: the
+// One CTA per (item, 64-wavenumber tile).  Bound by instruction latency: the
 // three contractions (FP32 FMAs) are a third of the instructions, the feature sums most of the rest,
 // and a warp waits 5 to 9 cycles between two of them.  So the design is for warps in flight and
 // few instructions: the path lengths once, packed (21 KB at 100 layers instead of 43), so that
@@ -238,8 +239,9 @@ k_adjoint_tile(AdjParams a) {
   __shared__ __align__(8) uint64_t bar;
   const FwdParams& p = a.f;
   // items fastest: the CTAs in flight share one tile's table rows in L2 (320 atmospheres on tables
-  // of 200,000 wavenumbers: 11.4 ms against 12.1 with the tiles fastest)
-  const int b = blockIdx.x, tile = blockIdx.y;          // tile: slot among the launched tiles
+  // of 200,000 wavenumbers: 11.4 ms against 12.1 with the tiles fastest).  Both in one dimension of
+  // the grid: a range of more than 4 million wavenumbers has more tiles than another can count
+  const int b = blockIdx.x % a.items, tile = blockIdx.x / a.items;   // tile: slot of the launch
   const bool jac = a.rows.n_rows > 0;
   const int wtile = jac ? a.rows.tile[tile] : tile;   // wavenumber tile
   const int jac_bin = jac ? a.rows.first_bin + a.rows.row[tile] : -1;
@@ -1333,10 +1335,10 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   auto backward = [&](int bc, const RowGroup& rows, int slots, double* grad,
                       long long stride) -> int {
     const int n_rows = std::max(rows.n_rows, 1);
-    ap.rows = rows; ap.tiles = slots;
+    ap.rows = rows; ap.tiles = slots; ap.items = (unsigned)bc;
     {
       KernelTimer kt(ctx, "k_adjoint_tile", s);
-      kern<<<dim3(bc, slots), kAThreads, smem, s>>>(ap);
+      kern<<<(unsigned)bc * (unsigned)slots, kAThreads, smem, s>>>(ap);
       err = cudaGetLastError();
     }
     if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint tile kernel: ") + cudaGetErrorString(err));
