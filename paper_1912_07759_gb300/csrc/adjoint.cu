@@ -63,7 +63,7 @@ struct AdjParams {
   const double* inv_dtc;          // [n_t_cia - 1]
   const float* gd;                // [B][n_in] dL/dD at the native wavenumbers of the range
   int n_in, tiles, n_feat;        // tiles: slots per item of the partial sums
-  unsigned items;                 // of the launch
+  int first_slot;                 // of the launch (the partial sums' pointers are its slot 0's)
   unsigned ray_mask;              // species with Rayleigh cross-sections that are not all zero
   float* part_a;                  // [B][tiles][npad]
   float* part_dl;                 // [B][tiles][npad][npad]  (ray j, shell l), j <= l
@@ -221,7 +221,7 @@ struct AdjSmem {
   }
 };
 
-// One CTA per (item, 64-wavenumber tile).  Bound by instruction latency: the
+// One CTA per (item, 64-wavenumber tile); grid (items, tiles).  Bound by instruction latency: the
 // three contractions (FP32 FMAs) are a third of the instructions, the feature sums most of the rest,
 // and a warp waits 5 to 9 cycles between two of them.  So the design is for warps in flight and
 // few instructions: the path lengths once, packed (21 KB at 100 layers instead of 43), so that
@@ -239,12 +239,12 @@ k_adjoint_tile(AdjParams a) {
   __shared__ __align__(8) uint64_t bar;
   const FwdParams& p = a.f;
   // items fastest: the CTAs in flight share one tile's table rows in L2 (320 atmospheres on tables
-  // of 200,000 wavenumbers: 11.4 ms against 12.1 with the tiles fastest).  Both in one dimension of
-  // the grid: a range of more than 4 million wavenumbers has more tiles than another can count
-  const int b = blockIdx.x % a.items, tile = blockIdx.x / a.items;   // tile: slot of the launch
+  // of 200,000 wavenumbers: 11.4 ms against 12.1 with the tiles fastest)
+  const int b = blockIdx.x, tile = blockIdx.y;            // tile: slot of the launch
+  const int slot = a.first_slot + tile;
   const bool jac = a.rows.n_rows > 0;
-  const int wtile = jac ? a.rows.tile[tile] : tile;   // wavenumber tile
-  const int jac_bin = jac ? a.rows.first_bin + a.rows.row[tile] : -1;
+  const int wtile = jac ? a.rows.tile[slot] : slot;   // wavenumber tile
+  const int jac_bin = jac ? a.rows.first_bin + a.rows.row[slot] : -1;
   const int N = p.buf.items[b].n_layers;
   if (N == 0) return;                                   // the item kernel zeroes its gradient
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -1301,8 +1301,7 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
     for (int m = 0; m < t->n_mol; ++m) ap.f.logsig_off[m] = t->logsig_offset[m];
   }
   ap.inv_dt = t->d_inv_dt; ap.inv_dtc = t->d_inv_dtc; ap.gd = gd; ap.n_in = n_in;
-  ap.n_feat = n_feat; ap.part_a = part_a; ap.part_dl = part_dl;
-  ap.part_f = part_f; ap.part_rp = part_rp;
+  ap.n_feat = n_feat;
   ap.kstore = use_kstore ? kbuf : nullptr;
   ap.kcols = forward_kcols(bins->dev.i0, n_in);
   ap.t_ptr = bins->dev.t_ptr; ap.t_bin = bins->dev.t_bin; ap.t_w = bins->dev.t_w;
@@ -1335,11 +1334,20 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
   auto backward = [&](int bc, const RowGroup& rows, int slots, double* grad,
                       long long stride) -> int {
     const int n_rows = std::max(rows.n_rows, 1);
-    ap.rows = rows; ap.tiles = slots; ap.items = (unsigned)bc;
+    ap.rows = rows; ap.tiles = slots;
     {
       KernelTimer kt(ctx, "k_adjoint_tile", s);
-      kern<<<(unsigned)bc * (unsigned)slots, kAThreads, smem, s>>>(ap);
-      err = cudaGetLastError();
+      // a range of more than 4 million wavenumbers has more tiles than the grid's second dimension
+      constexpr int kMaxY = 65535;
+      for (int s0 = 0; s0 < slots && err == cudaSuccess; s0 += kMaxY) {
+        ap.first_slot = s0;
+        ap.part_a = part_a + (size_t)s0 * npad;
+        ap.part_dl = part_dl + (size_t)s0 * npad * npad;
+        ap.part_f = part_f + (size_t)s0 * d->max_layers * n_feat;
+        ap.part_rp = part_rp + s0;
+        kern<<<dim3(bc, std::min(slots - s0, kMaxY)), kAThreads, smem, s>>>(ap);
+        err = cudaGetLastError();
+      }
     }
     if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, std::string("adjoint tile kernel: ") + cudaGetErrorString(err));
     if (slots > n_rows) {
