@@ -47,14 +47,13 @@ __device__ __forceinline__ int tix(int row, int c) {
   return row * kAT + ((((c >> 2) ^ (row >> 2)) & (kAT / 4 - 1)) << 2) + (c & 3);
 }
 
-// Jacobian rows done by one launch of each backward kernel: row r is bin first_bin + r, its tiles
-// are the slots [slot0[r], slot0[r + 1]).
-constexpr int kMaxRowSlots = 256;
+// Jacobian rows done by one launch of each backward kernel: row r is bin first_bin + r, its slots
+// [slot0[r], slot0[r + 1]) hold the wavenumber tiles from tile0[r] on.
+constexpr int kMaxRows = 256;        // bins of a gradient or Jacobian
 struct RowGroup {
   int n_rows, first_bin;
-  uint16_t slot0[kMaxRowSlots + 1];
-  int tile[kMaxRowSlots];
-  uint8_t row[kMaxRowSlots];
+  int slot0[kMaxRows + 1];
+  int tile0[kMaxRows];
 };
 
 struct AdjParams {
@@ -72,8 +71,7 @@ struct AdjParams {
   const float* kstore;            // the forward's K of the items, or NULL: recompute
   long long kcols;                // columns of a K row in kstore
   // rows.n_rows == 0: one gradient, slot = wavenumber tile, dL/dD from gd.  Else a group of
-  // Jacobian rows: slot s takes tile rows.tile[s] of bin rows.bin[s], dL/dD from that bin's
-  // weights (its row of dD_bin/dtheta)
+  // Jacobian rows: dL/dD of a row's slots from its bin's weights (its row of dD_bin/dtheta)
   RowGroup rows;
   const int* t_ptr; const int* t_bin; const double* t_w;   // the bins' transpose (BinsDev)
 };
@@ -241,10 +239,15 @@ k_adjoint_tile(AdjParams a) {
   // items fastest: the CTAs in flight share one tile's table rows in L2 (320 atmospheres on tables
   // of 200,000 wavenumbers: 11.4 ms against 12.1 with the tiles fastest)
   const int b = blockIdx.x, tile = blockIdx.y;            // tile: slot of the launch
-  const int slot = a.first_slot + tile;
   const bool jac = a.rows.n_rows > 0;
-  const int wtile = jac ? a.rows.tile[slot] : slot;   // wavenumber tile
-  const int jac_bin = jac ? a.rows.first_bin + a.rows.row[slot] : -1;
+  const int slot = a.first_slot + tile;
+  int row = 0;                                          // the last row whose slots begin at or before
+  for (int hi = a.rows.n_rows; row + 1 < hi;) {
+    const int mid = (row + hi) >> 1;
+    if (a.rows.slot0[mid] <= slot) row = mid; else hi = mid;
+  }
+  const int wtile = jac ? a.rows.tile0[row] + slot - a.rows.slot0[row] : slot;   // wavenumber tile
+  const int jac_bin = jac ? a.rows.first_bin + row : -1;
   const int N = p.buf.items[b].n_layers;
   if (N == 0) return;                                   // the item kernel zeroes its gradient
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
@@ -755,16 +758,6 @@ k_gd(BinsDev bd, int B, const double* __restrict__ binned, const double* __restr
   }
 }
 
-// gd of one Jacobian row: bin `bin`'s normalised weights.
-__global__ void k_row_gd(BinsDev bd, int bin, float* __restrict__ gd, int n_in) {
-  const int i = blockIdx.x * blockDim.x + threadIdx.x;
-  if (i >= n_in) return;
-  float g = 0.f;
-  for (int e = bd.t_ptr[i]; e < bd.t_ptr[i + 1]; ++e)
-    if (bd.t_bin[e] == bin) g = (float)bd.t_w[e];
-  gd[(size_t)blockIdx.y * n_in + i] = g;
-}
-
 // Sum of the wavenumber tiles' partial sums of one array [B][tiles][M] into its tile-0 slot,
 // in tile order (deterministic), compensated (Kahan) so the FP32 sum of hundreds of tiles
 // keeps about FP32 rounding; blockIdx.y picks the array.  Consecutive threads take
@@ -795,12 +788,19 @@ __global__ void k_adjoint_sum(TileSumArgs ts, int B) {
     if (tri > 0 && __all_sync(0xffffffffu, (int)m % tri < (int)m / tri)) continue;   // l < j
     float* row = arr + ((size_t)b * ts.slots + s0) * M + m;
     float s = row[0], c = 0.f;
-    for (int t = 1; t < tiles; ++t) {
+    auto add = [&](int t) {
       const float y = __fsub_rn(row[(size_t)t * M], c);
       const float u = __fadd_rn(s, y);
       c = __fsub_rn(__fsub_rn(u, s), y);
       s = u;
+    };
+    int t = 1;                                          // eight tiles' loads in flight
+    for (; t + 8 <= tiles; t += 8) {
+#pragma unroll
+      for (int k = 0; k < 8; ++k) add(t + k);
     }
+#pragma unroll 4
+    for (; t < tiles; ++t) add(t);
     row[0] = s;
   }
 }
@@ -1235,7 +1235,7 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
     return set_error(ctx, TR_ERR_UNSUPPORTED, "tables were loaded without FP32 storage");
   if (mixed && !t->d_logsig16 && t->n_mol > 0)
     return set_error(ctx, TR_ERR_UNSUPPORTED, "tables were loaded without FP16 log10 storage");
-  if (bins->dev.n_bin > 256) return set_error(ctx, TR_ERR_ARG, "the adjoint supports at most 256 bins");
+  if (bins->dev.n_bin > kMaxRows) return set_error(ctx, TR_ERR_ARG, "the adjoint supports at most 256 bins");
   if (t->interp_mode != TR_INTERP_LINEAR)
     return set_error(ctx, TR_ERR_UNSUPPORTED, "the adjoint implements the linear temperature scheme");
   if (d->t_profile != TR_TPROF_NPOINT || d->gas_mode != TR_GAS_CONSTANT)
@@ -1423,39 +1423,23 @@ extern "C" int tr_adjoint_transit(tr_ctx* ctx, const tr_tables* t, const tr_batc
     // bin's native range, so a row covers only the tiles of that range.  The rows go in groups
     // of as many as the partial sums' space for one gradient (`tiles` slots per item) holds, one
     // launch of each kernel per group: a launch per row left the GPU with one row's CTAs (128
-    // atmospheres, 50 bins of about 19 wavenumbers: 7.86 ms a call, in groups 2.3 ms).
+    // atmospheres, 50 bins of about 19 wavenumbers: 7.86 ms a call, in groups 2.3 ms).  Rows are
+    // described by their first tiles, so that a group can hold bins of any width (two atmospheres,
+    // four bins of about 19,000 wavenumbers: 0.71 ms a call with a launch per row, 0.33 in groups).
     const int base = wn_first(bins->dev.i0);
     const int n_bin = bins->dev.n_bin;
-    const int cap = std::min(tiles, kMaxRowSlots);
     auto first_tile = [&](int k) { return (bins->bin_lo[k] - base) / kAT; };
     auto n_tiles = [&](int k) { return (bins->bin_hi[k] - 1 - base) / kAT + 1 - first_tile(k); };
-    for (int k0 = 0; k0 < n_bin;) {
+    for (int k = 0; k < n_bin;) {
       RowGroup g;
-      g.n_rows = 0; g.first_bin = k0;
-      int slots = 0, k = k0;
-      for (; k < n_bin && slots + n_tiles(k) <= cap; ++k) {
-        g.slot0[g.n_rows] = (uint16_t)slots;
-        for (int q = 0; q < n_tiles(k); ++q, ++slots) {
-          g.tile[slots] = first_tile(k) + q;
-          g.row[slots] = (uint8_t)g.n_rows;
-        }
-        ++g.n_rows;
+      g.n_rows = 0; g.first_bin = k; g.slot0[0] = 0;
+      // at least one row: no bin has more tiles than the range
+      for (; k < n_bin && g.slot0[g.n_rows] + n_tiles(k) <= tiles; ++k, ++g.n_rows) {
+        g.tile0[g.n_rows] = first_tile(k);
+        g.slot0[g.n_rows + 1] = g.slot0[g.n_rows] + n_tiles(k);
       }
-      if (g.n_rows == 0) {
-        // a bin of more tiles than a group can list: its tiles one gradient-like pass, dL/dD
-        // written to gd
-        k_row_gd<<<dim3((n_in + 255) / 256, bc), 256, 0, s>>>(bins->dev, k, gd, n_in);
-        err = cudaGetLastError();
-        if (err != cudaSuccess) return set_error(ctx, TR_ERR_CUDA, cudaGetErrorString(err));
-        rc = backward(bc, g, tiles, jac + (size_t)k * nth, (long long)n_bin * nth);
-        if (rc != TR_OK) return rc;
-        k0 = k + 1;
-        continue;
-      }
-      g.slot0[g.n_rows] = (uint16_t)slots;
-      rc = backward(bc, g, slots, jac + (size_t)k0 * nth, (long long)n_bin * nth);
+      rc = backward(bc, g, g.slot0[g.n_rows], jac + (size_t)g.first_bin * nth, (long long)n_bin * nth);
       if (rc != TR_OK) return rc;
-      k0 = k;
     }
   }
   return TR_OK;
