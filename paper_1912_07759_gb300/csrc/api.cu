@@ -779,6 +779,7 @@ extern "C" int tr_make_bins(tr_ctx* ctx, const tr_tables* t, int n_bin, const do
   if (e == cudaSuccess) e = cudaMemcpy(m + o_lo, bin_lo.data(), sizeof(int) * n_bin, cudaMemcpyHostToDevice);
   if (e != cudaSuccess) { tr_free_bins(b); return cuda_fail(ctx, e, "copy bins"); }
   b->dev.n_bin = n_bin; b->dev.i0 = lo; b->dev.i1 = hi;
+  for (int j = 0; j < n_bin; ++j) b->dev.longest = std::max(b->dev.longest, row_ptr[j + 1] - row_ptr[j]);
   b->dev.row_ptr = reinterpret_cast<const int*>(m + o_row);
   b->dev.col = reinterpret_cast<const int*>(m + o_col);
   b->dev.w = reinterpret_cast<const double*>(m + o_w);

@@ -132,12 +132,24 @@ k_bin_group(BinsDev bd, long long n, const double* __restrict__ vals, long long 
 }
 
 // Several warps per bin while the batch is too small to fill the GPU with one per bin; eight lanes
-// per bin once these fill it (four warps on each of an SM's schedulers).
+// per bin once these fill it (four warps on each of an SM's schedulers) and no bin is so long that
+// its lanes wait for their loads one after the other.  Time by a warp per bin / by eight lanes, 8 to
+// 50 bins, without and with uncertainties: 8,192 bins of 800 entries 1.10 / 1.03, of 1,200 1.04 /
+// 1.00, of 1,500 0.84 / 0.92, of 8,000 0.79 / 0.87; 32,768 of 1,500 0.97 to 1.00 / 1.04, of 3,000
+// 0.90 / 0.98; 65,536, where the lanes fill the GPU's threads, of 3,000 1.03 / 1.04, of 8,000 0.97 /
+// 0.98.
+// Spectra of a single bin leave seven of a CTA's eight warps idle in the other form: 16,384 of
+// 1,500 1.24 / 1.05, of 6,000 1.16 / 0.96.  (Its grid counts spectra in the second dimension.)
+bool bin_by_groups(const BinsDev& bd, int B) {
+  const long long n = (long long)B * bd.n_bin;
+  if (n < 8192) return false;
+  return bd.longest <= (n >= 65536 ? 3072 : n >= 16384 ? 1600 : 1280) || (bd.n_bin == 1 && n >= 16384) || B > 65535;
+}
 template <int MODE>
 cudaError_t launch_bin_mode(const BinsDev& bd, int B, const double* vals, long long stride,
                             int base, double* out, cudaStream_t s) {
   const long long n = (long long)B * bd.n_bin;
-  if (n >= 8192) {
+  if (bin_by_groups(bd, B)) {
     constexpr int kPer = 32 * kBinWarps / kBinLanes;
     k_bin_group<MODE><<<(unsigned)((n + kPer - 1) / kPer), 32 * kBinWarps, 0, s>>>(
         bd, n, vals, stride, base, out);

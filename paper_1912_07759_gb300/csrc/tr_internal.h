@@ -302,6 +302,7 @@ cudaError_t launch_forward_fused(const FwdParams& p, const CUtensorMap* tm_sig,
 
 struct BinsDev {
   int n_bin, i0, i1;          // native range [i0, i1) with weight
+  int longest;                // entries of the longest bin
   const int* row_ptr;         // [n_bin + 1] into col/w
   const int* col;             // native index
   const double* w;            // weight w_ij
