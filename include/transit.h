@@ -336,8 +336,8 @@ int tr_forward_emission_batch(tr_ctx* ctx, const tr_tables* tables, const tr_bat
  * The batched forward of a sampler loop as one CUDA graph (the paper has no counterpart; its
  * retrievals evaluate the forward model once per live point, Sec. 6, and this packages that
  * repeated call).  Same arguments and outputs as tr_forward_transit_batch, plus:
- *   autotune: non-zero to time every configuration of the forward (two-stage form with 3, 2
- *     or 1 opacity CTAs per SM; for FP32 also the fused kernel) on these inputs first -- one
+ *   autotune: non-zero to time every configuration of the forward (two-stage form with as
+ *     many opacity CTAs per SM as fit, 2 or 1; for FP32 also the fused kernel) on these inputs first -- one
  *     warm-up and five timed runs each on `stream` -- and keep the fastest.  The choice is
  *     remembered on the context for this batch shape (tables, B, max_layers, precision,
  *     output range), so later captures and tr_forward_transit_batch calls of the same shape
@@ -370,7 +370,8 @@ int tr_graph_info(const tr_graph* graph, int* form, int* per_sm, int* stages,
 void tr_free_graph(tr_graph* graph);
 /* Set (pin) or forget the forward configuration the context uses for one batch shape (the
    autotuner's result, or a caller's choice): form 0 two-stage (per_sm opacity CTAs per SM,
-   0..3, 0 = as many as fit; contract_per_sm the FP32 contraction, 0..3 as in tr_graph_info;
+   0..3, 0 = as many as fit, which the linear temperature scheme's kernel is fastest with: up to
+   six; contract_per_sm the FP32 contraction, 0..3 as in tr_graph_info;
    3 on more than 112 layers is TR_ERR_UNSUPPORTED) or 1 fused FP32 kernel (stages: ring-depth cap, 0 = deepest).
    native: 1 for native-resolution output, 0 for the binned region of `bins`. */
 int tr_pin_forward_config(tr_ctx* ctx, const tr_tables* tables, const tr_batch_desc* desc,

@@ -86,9 +86,9 @@ __device__ __forceinline__ unsigned d_flags(int4 v) { return ((unsigned)v.z >> 1
 static_assert(offsetof(LayerDesc, flags) == 42 && offsetof(LayerDesc, tp) == 20,
               "layer descriptor offsets the header loads assume");
 
-// Packed FP32 pairs beyond ffma2 (sm_100 and later): pack2(lo, hi) forms the pair, unpack2
-// returns its halves; fma2, add2, sub2 and mul2 act on each half, rounded as the scalar
-// operation would be.
+// Packed FP32 pairs beyond ffma2 and fma2 (sm_100 and later): pack2(lo, hi) forms the pair, unpack2
+// returns its halves; add2, sub2 and mul2 act on each half, rounded as the scalar operation
+// would be.
 __device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
   unsigned long long r;
   asm("mov.b64 %0, {%1, %2};" : "=l"(r) : "f"(lo), "f"(hi));
@@ -97,12 +97,6 @@ __device__ __forceinline__ unsigned long long pack2(float lo, float hi) {
 __device__ __forceinline__ float2 unpack2(unsigned long long v) {
   float2 r;
   asm("mov.b64 {%0, %1}, %2;" : "=f"(r.x), "=f"(r.y) : "l"(v));
-  return r;
-}
-__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
-                                                   unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
   return r;
 }
 __device__ __forceinline__ unsigned long long add2(unsigned long long a, unsigned long long b) {

@@ -177,7 +177,7 @@ k_opacity_exp(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
     }
   };
   int seg = 0;
-  int cip = -1, cit = -1, citc = -1, czone = -1;
+  int cip = -1, cit = -1, citc = -1;
   float uc[2][2] = {};
   // per molecule, P row and wavenumber log2 sigma at T_j and its step
   // to T_j+1 (or, for pairs marked in `lin`, the linear values)
@@ -205,9 +205,9 @@ k_opacity_exp(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
     // 20,000 wavenumbers, 8 absorbers: 623 us, 566 so)
     const int row = (cur.o.bc * ((int)kcols / kKTile) + cur.o.tile * (kOT / kKTile) + c2 / kKTile) * p.max_layers + l0;
     float* dst = kbuf + (size_t)row * kKTile + col % kKTile;
-    if (l0 == cur.o.l_begin) cip = cit = citc = czone = -1;
-    const SegFlags f = segment_flags<false>(cur.h, l0, cur.o.l_begin, N, lane, has_mol, has_cia,
-                                            cip, cit, citc, czone);
+    if (l0 == cur.o.l_begin) cip = cit = citc = -1;
+    const SegFlags f = segment_flags(cur.h, l0, cur.o.l_begin, N, lane, has_mol, has_cia, cip,
+                                     cit, citc);
     const float4 ha = cur.ha, hb = cur.hb;
     const float ray0 = cur.ray.x, ray1 = cur.ray.y;
     const int n_here = min(32, N - l0);
@@ -285,17 +285,6 @@ int ring_stages(uint32_t stage_bytes, int ctas, uint32_t fixed) {
   const uint32_t per = kSmemPerSm / (uint32_t)ctas - 1024u - 512u;   // runtime reserve, statics
   const int s = per > fixed + 128u ? (int)((per - fixed - 128u) / sb) : 0;
   return std::max(2, std::min(s, kRingMaxStages));
-}
-
-// Layer blocks per (item, wavenumber tile) unit of the opacity kernel: 1 unless there are
-// fewer units than resident CTAs (a narrow wavenumber range of a few items), where splitting
-// the layers (blocks of at least 8) gives the idle CTAs work.  Measured on the full-size
-// single atmosphere (782 units, 456 CTAs), splitting to even out the last pass over the grid
-// costs more in repeated segment loads and unit start-up than it saves.
-int opacity_layer_blocks(long long units, long long slots, int max_layers) {
-  if (units <= 0 || 2 * units > slots) return 1;
-  const long long n = std::min<long long>(8, slots / units);
-  return (int)std::max<long long>(1, std::min<long long>(n, max_layers / 8));
 }
 
 int sm_count() {

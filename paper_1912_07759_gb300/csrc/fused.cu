@@ -152,7 +152,7 @@ k_forward_tma(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
       float xm[MAXMOL], yq[MAXCIA];
       item_weights<MAXMOL, MAXCIA>(p, b, 0, xm, yq);
       float us[4][2] = {}, uc[2][2] = {};
-      int cip = -1, cit = -1, citc = -1, czone = -1;
+      int cip = -1, cit = -1, citc = -1;
       bool mine = false;                             // the current segment is this group's
       for (int l0 = 0; l0 < N; l0 += 32) {
         const int li = l0 + lane;
@@ -163,17 +163,15 @@ k_forward_tma(FwdParams p, const __grid_constant__ CUtensorMap tm_sig,
           ha = __ldg(op + 2 * li);
           hb = __ldg(op + 2 * li + 1);
         }
-        const SegFlags f = segment_flags<false>(h, l0, 0, N, lane, has_mol, has_cia, cip, cit,
-                                                citc, czone);
+        const SegFlags f = segment_flags(h, l0, 0, N, lane, has_mol, has_cia, cip, cit, citc);
         const int n_here = min(32, N - l0);
         for (int i = 0; i < n_here; ++i) {
           if ((f.start >> i) & 1u) {
             mine = seg % kFOG == g;
             // the molecular cell or CIA bracket may carry over from earlier segments, which
             // other groups took: reload both sums for every segment this group takes
-            if (mine && !ring_consume<kFT, 2, MAXMOL, MAXCIA, false>(p, rs, plan, ring, seg,
-                                                                      has_mol, has_cia, c2, xm,
-                                                                      yq, us, uc, lane))
+            if (mine && !ring_consume<kFT, MAXMOL, MAXCIA>(p, rs, plan, ring, seg, has_mol,
+                                                            has_cia, c2, xm, yq, us, uc, lane))
               return;
             ++seg;
           }

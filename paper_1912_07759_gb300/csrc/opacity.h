@@ -68,38 +68,32 @@ __device__ __forceinline__ OpUnit op_unit(const FwdParams& p, long long u, int B
 }
 
 // Segment starts among the 32 layers l0 .. l0+31 of a unit's layer range [l_begin, l_end)
-// (lane i holds layer l0 + i's bracket header h = (ip, it, itc, chemistry zone)): bit i of
-// `start` is set when layer l0 + i begins a segment, of `mol` when its molecular cell or zone
-// differs from the layer before, of `cia` when its CIA bracket or zone does (a new zone
-// changes the molecule and pair weights of the sums).  (cip, cit, citc, czone) carry the
-// header of layer l0 - 1 in (-1 at the range start: everything is loaded there) and of the
-// chunk's last layer out.
-// ZONES = false compiles the zone comparison out (callers that only see zone 0).
+// (lane i holds layer l0 + i's bracket header h = (ip, it, itc)): bit i of `start` is set when
+// layer l0 + i begins a segment, of `mol` when its molecular cell differs from the layer before,
+// of `cia` when its CIA bracket does.  (cip, cit, citc) carry the header of layer l0 - 1 in (-1
+// at the range start: everything is loaded there) and of the chunk's last layer out.  The callers
+// serve constant mixing ratios only: no chemistry zones.
 struct SegFlags { unsigned start, mol, cia; };
-template <bool ZONES = true>
 __device__ __forceinline__ SegFlags segment_flags(const int4& h, int l0, int l_begin, int l_end,
                                                   int lane, bool has_mol, bool has_cia,
-                                                  int& cip, int& cit, int& citc, int& czone) {
+                                                  int& cip, int& cit, int& citc) {
   int pip = __shfl_up_sync(0xffffffffu, h.x, 1);
   int pit = __shfl_up_sync(0xffffffffu, h.y, 1);
   int pitc = __shfl_up_sync(0xffffffffu, h.z, 1);
-  int pzone = ZONES ? __shfl_up_sync(0xffffffffu, h.w, 1) : 0;
-  if (lane == 0) { pip = cip; pit = cit; pitc = citc; pzone = czone; }
+  if (lane == 0) { pip = cip; pit = cit; pitc = citc; }
   const int li = l0 + lane;
   const int N = l_end;
   const bool valid = li < N, first = li == l_begin;
-  const bool zchg = ZONES && h.w != pzone;
-  const bool mol = valid && has_mol && (first || h.x != pip || h.y != pit || zchg);
-  const bool cia = valid && has_cia && (first || h.z != pitc || zchg);
+  const bool mol = valid && has_mol && (first || h.x != pip || h.y != pit);
+  const bool cia = valid && has_cia && (first || h.z != pitc);
   SegFlags f;
-  f.start = __ballot_sync(0xffffffffu, valid && (mol || cia || first || zchg));
+  f.start = __ballot_sync(0xffffffffu, valid && (mol || cia || first));
   f.mol = __ballot_sync(0xffffffffu, mol);
   f.cia = __ballot_sync(0xffffffffu, cia);
   const int last = min(31, N - 1 - l0);
   cip = __shfl_sync(0xffffffffu, h.x, last);
   cit = __shfl_sync(0xffffffffu, h.y, last);
   citc = __shfl_sync(0xffffffffu, h.z, last);
-  if (ZONES) czone = __shfl_sync(0xffffffffu, h.w, last);
   return f;
 }
 
@@ -140,7 +134,7 @@ __device__ void ring_produce(const FwdParams& p, Ring& r, const RingPlan& plan,
   const int S = plan.stages;
   const bool has_mol = p.n_mol > 0, has_cia = p.n_cia > 0;
   const int wbase = wn_first(p.wn_begin);
-  int cip = -1, cit = -1, citc = -1, czone = -1;   // header carried into the next chunk read
+  int cip = -1, cit = -1, citc = -1;   // header carried into the next chunk read
   // first chunk of the first unit with layers at or after unit u
   auto first_from = [&](long long u, Chunk& c) -> bool {
     for (; u < n_units; u += gridDim.x) {
@@ -157,9 +151,9 @@ __device__ void ring_produce(const FwdParams& p, Ring& r, const RingPlan& plan,
     const LayerDesc* L = p.buf.layers + (size_t)(p.b_off + c.o.bc) * p.max_layers;
     const int li = c.l0 + lane;
     c.h = li < c.o.l_end ? __ldg(reinterpret_cast<const int4*>(L + li)) : make_int4(-1, -1, -1, 0);
-    if (c.l0 == c.o.l_begin) cip = cit = citc = czone = -1;
+    if (c.l0 == c.o.l_begin) cip = cit = citc = -1;
     c.f = segment_flags(c.h, c.l0, c.o.l_begin, c.o.l_end, lane, has_mol, has_cia, cip, cit,
-                        citc, czone);
+                        citc);
   };
   int seg = 0;
   bool stop = false;
@@ -213,18 +207,18 @@ __device__ void ring_produce(const FwdParams& p, Ring& r, const RingPlan& plan,
     }
 }
 
-// Consumer side of one segment start: waits for the stage (false: give up, the caller
-// returns), forms the sums over molecules us[c][v] = sum_m x_m sigma_m,c at the VW
-// wavenumbers col0 .. col0+VW-1 of the tile (corners c = (P_i,T_j) (P_i,T_j+1) (P_i+1,T_j)
-// (P_i+1,T_j+1)) when `mol`, and over CIA pairs uc[t][v] = sum_q y_q sigma_q,t when `cia`,
-// then releases the stage (one arrive per warp).
-template <int TW, int VW, int MAXMOL, int MAXCIA, bool F16>
+// Consumer side of one segment start (FP32 tables): waits for the stage (false: give up, the
+// caller returns), forms the sums over molecules us[c][v] = sum_m x_m sigma_m,c at the wavenumbers
+// col0 and col0 + 1 of the tile (corners c = (P_i,T_j) (P_i,T_j+1) (P_i+1,T_j) (P_i+1,T_j+1)) when
+// `mol`, and over CIA pairs uc[t][v] = sum_q y_q sigma_q,t when `cia`, then releases the stage
+// (one arrive per warp).  The sums are packed pairs (fma.rn.f32x2, each half rounded as fmaf in
+// the same order: the same values as scalar FMAs with half the instructions).
+template <int TW, int MAXMOL, int MAXCIA>
 __device__ __forceinline__ bool ring_consume(const FwdParams& p, Ring& r, const RingPlan& plan,
                                              const unsigned char* ring, int seg, bool mol,
                                              bool cia, int col0, const float* xm,
-                                             const float* yq, float (&us)[4][VW],
-                                             float (&uc)[2][VW], int lane) {
-  static_assert(VW == 1 || VW == 2, "one or two wavenumbers per lane");
+                                             const float* yq, float (&us)[4][2],
+                                             float (&uc)[2][2], int lane) {
   const int S = plan.stages;
   const int st = seg % S, k = seg / S;
   const bool ok = __all_sync(0xffffffffu, mbar_wait_bounded(&r.full[st], k & 1, p.dev_err,
@@ -232,106 +226,38 @@ __device__ __forceinline__ bool ring_consume(const FwdParams& p, Ring& r, const 
                                               !*(volatile int*)&r.abort_flag);
   if (!ok) { if (lane == 0) atomicExch(&r.abort_flag, 1); return false; }
   const unsigned char* sb = ring + st * plan.stage_bytes;
-  if constexpr (VW == 2 && !F16) {
-    // FP32 rows, two wavenumbers: the sums as packed pairs (fma.rn.f32x2, each half rounded as
-    // fmaf in the same order: the same values as scalar FMAs with half the instructions)
-    if (mol) {
-      unsigned long long x2[MAXMOL];
-#pragma unroll
-      for (int m = 0; m < MAXMOL; ++m) x2[m] = pack_dup(xm[m]);
-#pragma unroll
-      for (int c = 0; c < 4; ++c) {
-        unsigned long long s2 = 0ull;
-#pragma unroll
-        for (int m = 0; m < MAXMOL; ++m)
-          if (m < p.n_mol) {
-            const int e = (m * 4 + c) * TW + col0;   // box order: wn, T, P, molecule
-            ffma2(s2, x2[m], *reinterpret_cast<const unsigned long long*>(
-                                 reinterpret_cast<const float*>(sb) + e));
-          }
-        const float2 sum = *reinterpret_cast<const float2*>(&s2);
-        us[c][0] = sum.x;
-        us[c][1] = sum.y;
-      }
-    }
-    if (cia) {
-      const float* cbuf = reinterpret_cast<const float*>(sb + plan.mol_bytes);
-#pragma unroll
-      for (int t2 = 0; t2 < 2; ++t2) {
-        unsigned long long s2 = 0ull;
-#pragma unroll
-        for (int q = 0; q < MAXCIA; ++q)
-          if (q < p.n_cia)
-            ffma2(s2, pack_dup(yq[q]),
-                  *reinterpret_cast<const unsigned long long*>(cbuf + (2 * q + t2) * TW + col0));
-        const float2 sum = *reinterpret_cast<const float2*>(&s2);
-        uc[t2][0] = sum.x;
-        uc[t2][1] = sum.y;
-      }
-    }
-    __syncwarp();
-    if (lane == 0) mbar_arrive(&r.empty[st]);       // this warp is done with the stage
-    return true;
-  }
   if (mol) {
+    unsigned long long x2[MAXMOL];
+#pragma unroll
+    for (int m = 0; m < MAXMOL; ++m) x2[m] = pack_dup(xm[m]);
 #pragma unroll
     for (int c = 0; c < 4; ++c) {
-      float s[VW];
+      unsigned long long s2 = 0ull;
 #pragma unroll
-      for (int v = 0; v < VW; ++v) s[v] = 0.f;
-#pragma unroll
-      for (int m = 0; m < MAXMOL; ++m) {
+      for (int m = 0; m < MAXMOL; ++m)
         if (m < p.n_mol) {
-          const int e = (m * 4 + c) * TW + col0;   // box order: wn, T, P, molecule
-          float v[VW];
-          if constexpr (F16) {
-            const __half* hp = reinterpret_cast<const __half*>(sb) + e;
-            const float off = p.logsig_off[m];
-            if constexpr (VW == 2) {
-              const float2 hv = __half22float2(*reinterpret_cast<const __half2*>(hp));
-              v[0] = ex2_fast((hv.x + off) * kLog2Of10);
-              v[1] = ex2_fast((hv.y + off) * kLog2Of10);
-            } else {
-              v[0] = ex2_fast((__half2float(*hp) + off) * kLog2Of10);
-            }
-          } else {
-            const float* fp = reinterpret_cast<const float*>(sb) + e;
-            if constexpr (VW == 2) {
-              const float2 fv = *reinterpret_cast<const float2*>(fp);
-              v[0] = fv.x; v[1] = fv.y;
-            } else {
-              v[0] = *fp;
-            }
-          }
-#pragma unroll
-          for (int q = 0; q < VW; ++q) s[q] = fmaf(xm[m], v[q], s[q]);
+          const int e = (m * 4 + c) * TW + col0;     // box order: wn, T, P, molecule
+          ffma2(s2, x2[m], *reinterpret_cast<const unsigned long long*>(
+                               reinterpret_cast<const float*>(sb) + e));
         }
-      }
-#pragma unroll
-      for (int v = 0; v < VW; ++v) us[c][v] = s[v];
+      const float2 sum = *reinterpret_cast<const float2*>(&s2);
+      us[c][0] = sum.x;
+      us[c][1] = sum.y;
     }
   }
   if (cia) {
     const float* cbuf = reinterpret_cast<const float*>(sb + plan.mol_bytes);
 #pragma unroll
-    for (int t = 0; t < 2; ++t) {
-      float s[VW];
+    for (int t2 = 0; t2 < 2; ++t2) {
+      unsigned long long s2 = 0ull;
 #pragma unroll
-      for (int v = 0; v < VW; ++v) s[v] = 0.f;
-#pragma unroll
-      for (int q = 0; q < MAXCIA; ++q) {
-        if (q < p.n_cia) {
-          const float* fp = cbuf + (2 * q + t) * TW + col0;
-          if constexpr (VW == 2) {
-            const float2 fv = *reinterpret_cast<const float2*>(fp);
-            s[0] = fmaf(yq[q], fv.x, s[0]); s[1] = fmaf(yq[q], fv.y, s[1]);
-          } else {
-            s[0] = fmaf(yq[q], *fp, s[0]);
-          }
-        }
-      }
-#pragma unroll
-      for (int v = 0; v < VW; ++v) uc[t][v] = s[v];
+      for (int q = 0; q < MAXCIA; ++q)
+        if (q < p.n_cia)
+          ffma2(s2, pack_dup(yq[q]),
+                *reinterpret_cast<const unsigned long long*>(cbuf + (2 * q + t2) * TW + col0));
+      const float2 sum = *reinterpret_cast<const float2*>(&s2);
+      uc[t2][0] = sum.x;
+      uc[t2][1] = sum.y;
     }
   }
   __syncwarp();

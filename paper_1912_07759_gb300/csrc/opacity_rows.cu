@@ -129,13 +129,6 @@ __device__ __forceinline__ void row_pairs(const unsigned char* row, int g, int l
   }
 }
 
-__device__ __forceinline__ unsigned long long fma2_of(unsigned long long a, unsigned long long b,
-                                                      unsigned long long c) {
-  unsigned long long r;
-  asm("fma.rn.f32x2 %0, %1, %2, %3;" : "=l"(r) : "l"(a), "l"(b), "l"(c));
-  return r;
-}
-
 // Bytes of a ring stage: two rows of every molecule, one of every CIA pair.
 struct RowStage {
   unsigned mol, cia, bytes;
@@ -327,7 +320,7 @@ k_opacity_rows(FwdParams p, const __grid_constant__ CUtensorMap tm_t,
       unsigned long long kk[V2];
 #pragma unroll
       for (int i = 0; i < V2; ++i) {
-        kk[i] = fma2_of(rk.x, ray[i], rk.y);
+        kk[i] = fma2(rk.x, ray[i], rk.y);
         ffma2(kk[i], w01.x, us[0][i]);
         ffma2(kk[i], w01.y, us[1][i]);
         ffma2(kk[i], w23.x, us[2][i]);
@@ -351,15 +344,6 @@ k_opacity_rows(FwdParams p, const __grid_constant__ CUtensorMap tm_t,
   }
 }
 
-// Layer blocks per (item, wavenumber tile): 1 unless the units leave warps' places free (a
-// narrow range or few items), where the layers are split (blocks of at least 8) so that more
-// warps run; a block begins with four rows instead of two.
-int row_layer_blocks(long long units, long long slots, int max_layers) {
-  if (units <= 0 || 2 * units > slots) return 1;
-  const long long n = std::min<long long>(8, slots / units);
-  return (int)std::max<long long>(1, std::min<long long>(n, max_layers / 8));
-}
-
 template <int NMOL, int NCIA, bool ANY, bool F16>
 cudaError_t launch_t(const FwdParams& p, const RowMaps& tm, int Bc, float* kbuf, long long kcols,
                      int cap, cudaStream_t s) {
@@ -371,7 +355,7 @@ cudaError_t launch_t(const FwdParams& p, const RowMaps& tm, int Bc, float* kbuf,
   cudaGetDevice(&dev);
   cudaDeviceGetAttribute(&n_sm, cudaDevAttrMultiProcessorCount, dev);
   const long long units0 = (long long)Bc * groups;
-  const int n_lb = row_layer_blocks(units0, 4LL * std::max(n_sm, 1), p.max_layers);
+  const int n_lb = opacity_layer_blocks(units0, 4LL * std::max(n_sm, 1), p.max_layers);
   const int lb_size = (p.max_layers + n_lb - 1) / n_lb;
   const long long ctas = units0 * n_lb;
   if (ctas > 0x7fffffffLL) return cudaErrorInvalidValue;

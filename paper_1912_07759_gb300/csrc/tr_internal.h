@@ -173,6 +173,11 @@ __device__ __forceinline__ void ffma2(unsigned long long& acc, unsigned long lon
                                       unsigned long long b) {
   asm("fma.rn.f32x2 %0, %1, %2, %0;" : "+l"(acc) : "l"(a), "l"(b));
 }
+__device__ __forceinline__ unsigned long long fma2(unsigned long long a, unsigned long long b,
+                                                   unsigned long long c) {
+  ffma2(c, a, b);
+  return c;
+}
 #endif
 constexpr int kOpxStride = 16;   // floats of per-item opacity weights (TR_MAX_MOL + TR_MAX_CIA, padded)
 // Chemistry zones of a two-layer atmosphere: runs of layers with the same mixing ratios.  Each
@@ -215,8 +220,8 @@ cudaError_t launch_geometry(const GeomParams& gp, int B, const double* d_theta, 
 // tiles of every forward and adjoint kernel start here.
 __host__ __device__ inline int wn_first(int wn_begin) { return wn_begin & ~7; }
 
-// Wavenumbers per CTA of the TMA-staged opacity kernel (one per thread): the inner box size of
-// the tables' tensor maps.
+// Wavenumbers per CTA of the exponential scheme's opacity kernel (two per consumer lane): the inner
+// box size of the tables' tensor maps.
 constexpr int kOpacityTile = 256;
 // Wavenumbers per warp of the linear scheme's opacity kernel.
 constexpr int kRowTile = 256;
@@ -261,10 +266,21 @@ struct KSplit { int items, cols; };
 KSplit forward_split(int B, int max_layers, int wn_begin, int wn_count);
 // Opacity of items [p.b_off, p.b_off + Bc): FP32 tables, or the FP16 log tables when
 // p.logsig16 is set (decoded on the fly); t: the tables, for their tensor maps.
-// per_sm_cap: at most this many CTAs per SM (0: up to 3, as registers allow); the ring of
-// each takes the shared memory the others leave.
+// per_sm_cap: at most this many CTAs per SM (0: as many as fit, up to 6, with the exponential
+// scheme 3); the rings of each take the shared memory the others leave.
 cudaError_t launch_opacity(const FwdParams& p, const tr_tables* t, int Bc, float* kbuf,
                            int per_sm_cap, cudaStream_t s);
+// Layer blocks per (item, wavenumber tile) unit of an opacity kernel: 1 unless the units leave
+// half of the places for CTAs (or warps' tiles) free, a narrow range or few items, where the layers
+// are split (blocks of at least 8) to give the idle ones work.  Each block loads its first rows
+// anew: splitting to even out the last pass over the grid costs more than it saves (measured on
+// the full-size single atmosphere, 782 units for 456 CTAs).
+inline int opacity_layer_blocks(long long units, long long slots, int max_layers) {
+  if (units <= 0 || 2 * units > slots) return 1;
+  const long long n = slots / units, most = max_layers / 8;
+  const long long b = n < 8 ? n : 8;
+  return (int)(b < most ? b : most > 1 ? most : 1);
+}
 // The same with the linear temperature scheme (opacity_rows.cu), which launch_opacity takes.
 // Tensor maps with the inner box kRowTile wavenumbers: sigma boxes of two T rows at one P and of
 // two P rows at one T of every molecule, CIA boxes of one T row of every pair.
