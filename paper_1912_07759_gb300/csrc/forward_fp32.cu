@@ -555,6 +555,7 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
 
   // ---------------- contraction warps
   const int n_items = n_units * rt_max;
+  int landed = -1;                                      // the item whose path lengths it waited for last
   while (true) {
     int it = 0;
     if (lane == 0) it = atomicAdd(&next_item, 1);
@@ -577,16 +578,19 @@ k_contract_fp32(FwdParams p, const __grid_constant__ CUtensorMap tm_k, int Bc, i
     // k - kMaxSlots.  K of unit k has landed, so the producer has seen every unit up to k - S done,
     // that one among them.  (Two barriers are too few: with one unit per item and S = 3, three items
     // are in flight, and a wait for the third returns at once while the first one's path lengths are
-    // still arriving.)  The next phase starts only when every unit of this item is done
+    // still arriving.)  The next phase starts only when every unit of this item is done; a warp
+    // that has waited for the item does not ask again
     const int item = bc - u_begin / n_tiles;
     const bool ok = __all_sync(0xffffffffu, wait_slot(&slot_unit[sl], k, &abort_flag, p.dev_err) &&
                                                 mbar_wait_bounded(&kfull[sl], q & 1, p.dev_err,
                                                                   TR_DEVERR_TIMEOUT) &&
-                                                mbar_wait_bounded(&dlfull[item % kMaxSlots],
-                                                                  (item / kMaxSlots) & 1, p.dev_err,
-                                                                  TR_DEVERR_TIMEOUT) &&
+                                                (item == landed ||
+                                                 mbar_wait_bounded(&dlfull[item % kMaxSlots],
+                                                                   (item / kMaxSlots) & 1, p.dev_err,
+                                                                   TR_DEVERR_TIMEOUT)) &&
                                                 !*(volatile int*)&abort_flag);
     if (!ok) { if (lane == 0) atomicExch(&abort_flag, 1); return; }
+    landed = item;
     float* part = reinterpret_cast<float*>(base + sl * lay.slot + lay.ktb);
     if (N > 0) {
       float pt[4];
